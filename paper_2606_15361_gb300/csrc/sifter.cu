@@ -1225,15 +1225,37 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   }
 }
 
-// One block per snippet: 64 x 256 plane cells around (row, col), standardised with the FP64
-// mean and population std of the present cells (std 0 -> 1); missing cells are 0.
-__global__ void __launch_bounds__(256) k_snippets(const float* __restrict__ plane, long long ld, int ndm,
-                                                  long long ncols, const int32_t* __restrict__ rows,
-                                                  const int64_t* __restrict__ cols, int n, float* __restrict__ out) {
-  const int s = blockIdx.x;
-  if (s >= n) return;
-  const int r0 = rows[s] - 32;
-  const long long c0 = cols[s] - 128;
+// (h, l) + x as an unevaluated FP32 pair: h + l keeps about 48 bits of a sum (error-free two-sum)
+__device__ __forceinline__ void pair_add(float& h, float& l, float x) {
+  const float s = __fadd_rn(h, x);
+  const float t = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(x, t)));
+  h = s;
+}
+
+// The 256 threads' pairs summed: every thread of warp 0 gets the total (FP64), after a barrier.
+__device__ __forceinline__ double pair_sum_cta(float h, float l, float2* part) {
+  auto fold = [&](int o) {
+    const float oh = __shfl_xor_sync(0xFFFFFFFFu, h, o), ol = __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    pair_add(h, l, oh);
+    l = __fadd_rn(l, ol);
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) fold(o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(h, l);
+  __syncthreads();
+  if (threadIdx.x >= 32) return 0.0;
+  h = part[threadIdx.x & 7].x;
+  l = part[threadIdx.x & 7].y;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) fold(o);
+  return static_cast<double>(h) + static_cast<double>(l);
+}
+
+// A snippet wholly in FP64, for the value ranges the FP32 pairs do not cover (NaN, infinities,
+// a deviation of 0 or outside 1e-12 .. 1e15, means above 1e15).
+__device__ __noinline__ void snippet_fp64(const float* __restrict__ plane, long long ld, int ndm, long long ncols,
+                                          int r0, long long c0, float* __restrict__ o) {
   double s1 = 0.0, s2 = 0.0;
   long long cnt = 0;
   for (int i = threadIdx.x; i < kH * kW; i += blockDim.x) {
@@ -1249,10 +1271,10 @@ __global__ void __launch_bounds__(256) k_snippets(const float* __restrict__ plan
   __shared__ double r1[8], r2[8];
   __shared__ long long rc[8];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, o);
-    s2 += __shfl_xor_sync(0xFFFFFFFFu, s2, o);
-    cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
+  for (int o2 = 16; o2 > 0; o2 >>= 1) {
+    s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, o2);
+    s2 += __shfl_xor_sync(0xFFFFFFFFu, s2, o2);
+    cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o2);
   }
   if ((threadIdx.x & 31) == 0) {
     r1[threadIdx.x >> 5] = s1;
@@ -1270,7 +1292,6 @@ __global__ void __launch_bounds__(256) k_snippets(const float* __restrict__ plan
   const double mu = cnt ? s1 / cnt : 0.0;
   const double var = cnt ? s2 / cnt - mu * mu : 0.0;
   const double sd = var > 0.0 ? sqrt(var) : 1.0;
-  float* o = out + static_cast<long long>(s) * kH * kW;
   for (int i = threadIdx.x; i < kH * kW; i += blockDim.x) {
     const int r = r0 + i / kW;
     const long long c = c0 + (i % kW);
@@ -1278,6 +1299,97 @@ __global__ void __launch_bounds__(256) k_snippets(const float* __restrict__ plan
     if (r >= 0 && r < ndm && c >= 0 && c < ncols)
       v = static_cast<float>((plane[static_cast<long long>(r) * ld + c] - mu) / sd);
     o[i] = v;
+  }
+}
+
+// One CTA per snippet: 64 x 256 plane cells around (row, col), standardised with the mean and
+// population std of the present cells (std 0 -> 1); missing cells are 0. A thread keeps one
+// column's 64 cells in registers, so the plane is read once, and with 64 loads in flight a
+// thread. The FP64 pipe of this chip runs 1/64 of the FP32 rate, so an FP64 evaluation per cell
+// bounds a kernel that should be bound by its stores: the sums, the differences v - mu and the
+// products with 1 / sd are unevaluated FP32 pairs (two-sum, two-product: about 48 bits, so the
+// rounded result is the FP64 one), FP64 only in one warp, for the
+// CTA's two totals. The deviations are summed
+// about the mean, not as s2 / n - mu^2. 4096 snippets
+// of a 2048 x 16384 plane take 200 us (64: 13 us); with FP64 sums and divisions per cell 1806 us
+// (64: 72 us). What is left is latency: two CTAs fit an SM (the cells in registers), and each
+// loads, reduces twice and stores one after the other; the bytes alone would take about 80 us.
+__global__ void __launch_bounds__(256, 2) k_snippets(const float* __restrict__ plane, long long ld, int ndm,
+                                                     long long ncols, const int32_t* __restrict__ rows,
+                                                     const int64_t* __restrict__ cols, int n,
+                                                     float* __restrict__ out) {
+  __shared__ float2 part1[8], part2[8];
+  __shared__ float2 mean2, inv2;  // the mean and 1 / sd as pairs (inv2.x = 0: the FP64 path)
+  static_assert(kW == 256, "one thread per column");
+  const int s = blockIdx.x, tx = threadIdx.x;
+  if (s >= n) return;
+  const int r0 = rows[s] - 32;
+  const long long c0 = cols[s] - 128;
+  float* o = out + static_cast<long long>(s) * kH * kW;
+  const long long c = c0 + tx;
+  const bool cok = c >= 0 && c < ncols;
+  const int lo = r0 < 0 ? min(-r0, kH) : 0, hi = r0 + kH > ndm ? max(ndm - r0, 0) : kH;  // present rows [lo, hi)
+  const long long clo = c0 < 0 ? 0 : c0, chi = c0 + kW > ncols ? ncols : c0 + kW;
+  const double cnt = hi > lo && chi > clo ? static_cast<double>((hi - lo) * (chi - clo)) : 0.0;
+  float v[kH];
+  const float* src = plane + static_cast<long long>(r0) * ld + c;
+#pragma unroll
+  for (int i = 0; i < kH; ++i) v[i] = cok && i >= lo && i < hi ? __ldg(src + static_cast<long long>(i) * ld) : 0.0f;
+  float h[4], l[4];  // four chains
+#pragma unroll
+  for (int k = 0; k < 4; ++k) h[k] = l[k] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kH; ++i) pair_add(h[i & 3], l[i & 3], v[i]);
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    pair_add(h[0], l[0], h[k]);
+    l[0] = __fadd_rn(l[0], l[k]);
+  }
+  const double sum = pair_sum_cta(h[0], l[0], part1);
+  if (tx == 0) {
+    const double mu = cnt > 0.0 ? sum / cnt : 0.0;
+    mean2.x = static_cast<float>(mu);
+    mean2.y = static_cast<float>(mu - static_cast<double>(mean2.x));
+  }
+  __syncthreads();
+  const float mh = mean2.x, ml = mean2.y;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) h[k] = l[k] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kH; ++i) {
+    if (!(cok && i >= lo && i < hi)) continue;
+    const float d = __fsub_rn(v[i], mh), t = __fsub_rn(d, v[i]);
+    const float e = __fsub_rn(__fsub_rn(__fsub_rn(v[i], __fsub_rn(d, t)), __fadd_rn(mh, t)), ml);  // v - mu = d + e
+    const float p = __fmul_rn(d, d);
+    pair_add(h[i & 3], l[i & 3], p);
+    // (d + e)^2 = p + (d^2 - p) + e (2 d + e)
+    l[i & 3] = __fadd_rn(l[i & 3], __fmaf_rn(__fadd_rn(__fadd_rn(d, d), e), e, __fmaf_rn(d, d, -p)));
+  }
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    pair_add(h[0], l[0], h[k]);
+    l[0] = __fadd_rn(l[0], l[k]);
+  }
+  const double ss = pair_sum_cta(h[0], l[0], part2);
+  if (tx == 0) {
+    const bool fits = fabsf(mh) <= 1e15f && ss >= 1e-24 * cnt && ss <= 1e30 * cnt && cnt > 0.0;  // false on NaN
+    const double inv = fits ? sqrt(cnt / ss) : 0.0;
+    inv2.x = static_cast<float>(inv);
+    inv2.y = static_cast<float>(inv - static_cast<double>(inv2.x));
+  }
+  __syncthreads();
+  const float rh = inv2.x, rl = inv2.y;
+  if (rh == 0.0f) {
+    snippet_fp64(plane, ld, ndm, ncols, r0, c0, o);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < kH; ++i) {
+    const float d = __fsub_rn(v[i], mh), t = __fsub_rn(d, v[i]);
+    const float e = __fsub_rn(__fsub_rn(__fsub_rn(v[i], __fsub_rn(d, t)), __fadd_rn(mh, t)), ml);
+    const float p = __fmul_rn(d, rh);
+    const float q = __fadd_rn(p, __fmaf_rn(e, rh, __fmaf_rn(d, rl, __fmaf_rn(d, rh, -p))));
+    o[i * kW + tx] = cok && i >= lo && i < hi ? q : 0.0f;
   }
 }
 
