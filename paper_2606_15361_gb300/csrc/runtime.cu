@@ -155,6 +155,9 @@ extern "C" int snd_bind_workspace(snd_plan_t plan, void* d_ws, size_t bytes, voi
   dp.ztab = z ? at<void>(d_ws, o.ztab) : nullptr;
   dp.zwb = z ? at<int32_t>(d_ws, o.zwb) : nullptr;
   dp.zcarry = z ? at<int32_t>(d_ws, o.zcarry) : nullptr;
+  dp.zeoff = z ? at<int32_t>(d_ws, o.zeoff) : nullptr;
+  dp.zent = z ? at<int32_t>(d_ws, o.zent) : nullptr;
+  dp.zdm = z ? at<uint32_t>(d_ws, o.zdm) : nullptr;
   std::vector<float> dmf(p.dms.begin(), p.dms.end());
   // uploads still in flight target the previous workspace
   if (p.up_stream && cudaStreamSynchronize(p.up_stream) != cudaSuccess) {
@@ -176,6 +179,9 @@ extern "C" int snd_bind_workspace(snd_plan_t plan, void* d_ws, size_t bytes, voi
   if (e == cudaSuccess) e = upload(d_ws, o.dbase, p.dbase, s);
   if (e == cudaSuccess && z) e = upload(d_ws, o.zwb, p.zwb, s);
   if (e == cudaSuccess && z) e = upload(d_ws, o.zcarry, p.zcarry, s);
+  if (e == cudaSuccess && z) e = upload(d_ws, o.zeoff, p.zeoff, s);
+  if (e == cudaSuccess && z) e = upload(d_ws, o.zent, p.zent, s);
+  if (e == cudaSuccess && z) e = upload(d_ws, o.zdm, p.zdm, s);
   if (e != cudaSuccess) {
     p.bound = false;
     return SND_ERR_CUDA;

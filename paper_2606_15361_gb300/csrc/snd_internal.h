@@ -109,7 +109,25 @@ struct ZGeom {
   int group_leaves;   // leaves staged per shared-memory round
   int smem_bytes;
   int Rz;             // payload ring samples per channel
+  // pattern-sharing form (see ztree.cu): each distinct leaf pattern of a DM tile summed once
+  int shared = 0;     // the plan uses it
+  int spread = 0;     // largest delay spread of a channel over a DM tile (samples)
+  int sspread = 0;    // largest spread of the leaf delays that one pattern serves (samples)
+  int share_pct = 0;  // patterns per (tile, leaf), times 100
+  std::vector<int> group_max;  // [G - 1]: most patterns of G consecutive leaves (from a multiple of G)
 };
+
+// Launch shape of the pattern-sharing labelled-payload tree for `np` pair slots per lane.
+struct ZShape {
+  int np;       // 64 np output samples per CTA
+  int win;      // staged payload samples per channel
+  int stride;   // samples of one stored pattern series
+  int group;    // leaves per shared-memory round (0: does not fit)
+  int smem;     // dynamic shared memory
+};
+ZShape ztree_shape(const struct Plan& p, int np);
+int ztree_max_pairs(int nlev);  // most and fewest pair slots per lane of the kernels for trees of nlev levels
+int ztree_min_pairs(int nlev);
 
 // Device pointers inside the bound workspace.
 struct DevPtrs {
@@ -147,6 +165,9 @@ struct DevPtrs {
   void* ztab;              // zfloat: [nchan][256] payload of each uint8 value (0 below the level)
   int32_t* zwb;            // zfloat: [ndm_tiles][nchan] first staged sample offset per channel
   int32_t* zcarry;         // zfloat: [nleaves] carry depth of each leaf
+  int32_t* zeoff;          // zfloat: [ndm_tiles][nleaves + 1] first pattern of each (tile, leaf)
+  int32_t* zent;           // zfloat: [patterns][8] window offset of each channel | (its first delay mod 8) << 28; [7]: leaf << 16 | span
+  uint32_t* zdm;           // zfloat: [ndm_tiles][nleaves][16] pattern in the tile << 14 | delay past the pattern's first
   uint16_t* dmeta;         // direct tree: [ndm_tiles][nchan][32] staged word offset << 5 | shift
   int32_t* dbase;          // direct tree: [ndm_tiles][nchan] first staged ring word (multiple of 4)
   unsigned long long* level_fires;  // [kMaxLevels] firing node-samples per tree level (SND_FLAG_LEVEL_RATES)
@@ -201,7 +222,8 @@ struct Plan {
   std::vector<uint16_t> dmeta;
   std::vector<int32_t> dbase;
   ZGeom zgeom{};
-  std::vector<int32_t> zwb, zcarry;
+  std::vector<int32_t> zwb, zcarry, zeoff, zent;
+  std::vector<uint32_t> zdm;
 
   // sizes
   int R = 0;           // ring words per copy
@@ -211,7 +233,7 @@ struct Plan {
   struct Off {
     size_t ring, hist, levels, plane, mask, mask2, mask3, cells, counters, row_runs, run_start,
         run_end, run_row, parent, npix, peak, pwidth, bcand, cand, staging, staging2, width_mask, dm_f32, tp_off,
-        gepk, gleaf, gmeta, tile_wb, delays, zring, ztab, zwb, zcarry, dmeta, dbase, level_fires;
+        gepk, gleaf, gmeta, tile_wb, delays, zring, ztab, zwb, zcarry, zeoff, zent, zdm, dmeta, dbase, level_fires;
   } off{};
 
   // binding and stream state
