@@ -283,7 +283,8 @@ int build_plan(Plan& p) {
   int rc = (p.mode == SND_MODE_ZFLOAT) ? choose_ztree_geometry(p) : choose_tree_geometry(p);
   if (p.mode != SND_MODE_ZFLOAT) {
     choose_direct_geometry(p);
-    if (p.direct) rc = SND_OK;  // the leaf-sharing kernel may not fit; the direct one does
+    // channel counts in whole groups: the leaf-sharing kernel may not fit, the direct one does
+    if (p.direct && p.dgeom.whole) rc = SND_OK;
   }
   if (rc) return rc;
 
@@ -301,7 +302,7 @@ int build_plan(Plan& p) {
     o = align_up(o + bytes, 256);
     return at;
   };
-  p.off.ring = take(sizeof(uint32_t) * static_cast<size_t>(nchan) * 2 * p.R);
+  p.off.ring = take(sizeof(uint32_t) * static_cast<size_t>(std::max(nchan, p.direct ? p.dgeom.nchan : 0)) * 2 * p.R);
   p.off.hist = take(sizeof(uint32_t) * static_cast<size_t>(nchan) * 256);
   p.off.levels = take(sizeof(int32_t) * nchan);
   p.off.plane = take(sizeof(int32_t) * static_cast<size_t>(ndm) * p.Lp);
@@ -529,7 +530,14 @@ void choose_direct_geometry(Plan& p) {
   p.dbase.clear();
   if (p.mode == SND_MODE_ZFLOAT || (p.flags & (SND_FLAG_REFERENCE_TREE | SND_FLAG_LEAF_SHARING))) return;
   const int nchan = p.nchan, ndm = p.ndm;
-  if (nchan % 64 != 0 || nchan >= 8192) return;
+  // the kernel adds 64 channels at a time: channels from nchan up to the next multiple are ring rows
+  // that stay zero (a channel that never fires changes no sum and no quorum). Adding them costs less
+  // than the leaf-sharing kernel at every count: tree us per 8192 samples x 512 DMs, direct /
+  // leaf-sharing, graded B = 8: 8 channels 17 / 23, 65 19 / 52, 140 23 / 58, 300 30 / 93, 1000 58 / 207.
+  const int nc = static_cast<int>(align_up(nchan, 64));
+  const bool rates = (p.flags & SND_FLAG_LEVEL_RATES) != 0;
+  if (nc >= 8192 || (rates && nc != nchan)) return;
+  g.whole = nc == nchan;
   int inst = snd::kDirNone, kw = 4;
   if (p.mode == SND_MODE_FLOAT) {
     inst = nchan < 2048 ? snd::kDirFloat11 : snd::kDirFloat13;
@@ -547,7 +555,11 @@ void choose_direct_geometry(Plan& p) {
     int64_t sub_ch = p.C;
     for (int l = 0; l < sub; ++l) sub_ch *= p.B;
     if (sub == p.nlev - 1) sub_ch = nchan;
-    if (sub_ch % 64 != 0 || nchan % sub_ch != 0) return;
+    // an exact-level node is whole 64-channel groups, but the last one, which ends with the channels
+    const bool root = sub_ch == nchan;
+    if (!root && sub_ch % 64 != 0) return;
+    g.whole = g.whole && sub_ch % 64 == 0 && nchan % sub_ch == 0;
+    if (rates && !g.whole) return;
     int planes = 0;
     while ((int64_t(1) << planes) <= sub_ch) ++planes;
     const int up = p.nlev - 1 - sub;
@@ -562,7 +574,7 @@ void choose_direct_geometry(Plan& p) {
       return;
     }
     g.sub_lev = sub;
-    g.sub_groups = static_cast<int>(sub_ch / 64);
+    g.sub_groups = static_cast<int>((sub_ch + 63) / 64);
   } else {
     if (p.C != 4 || p.KL < 1 || p.KL > 4 || p.KI < 1 || p.KI > 2 || p.nlev < 2) return;
     const int up = p.nlev - 1;
@@ -602,7 +614,7 @@ void choose_direct_geometry(Plan& p) {
     span_kw = std::max(kw, g.rates_kw);
   }
   g.ndm_tiles = (ndm + 31) / 32;
-  p.dbase.assign(static_cast<size_t>(g.ndm_tiles) * nchan, 0);
+  p.dbase.assign(static_cast<size_t>(g.ndm_tiles) * nc, 0);
   int64_t omax = 0;
   for (int t = 0; t < g.ndm_tiles; ++t)
     for (int c = 0; c < nchan; ++c) {
@@ -613,34 +625,35 @@ void choose_direct_geometry(Plan& p) {
         hi = std::max(hi, v);
       }
       const int32_t b4 = (lo >> 5) & ~3;
-      p.dbase[static_cast<size_t>(t) * nchan + c] = b4;
+      p.dbase[static_cast<size_t>(t) * nc + c] = b4;
       omax = std::max<int64_t>(omax, (hi >> 5) - b4);
     }
   if (omax > 2047) return;
   g.cspan = static_cast<int>(align_up(static_cast<size_t>(4 + omax + g.warps * span_kw), 4));
   // stage 128 channels per round (half the barriers) when they fit two CTAs per SM
-  auto smem_for = [&](int sg) { return (2 * 64 * sg * static_cast<int64_t>(g.cspan) + 64 * sg * 32 + nchan) * 4; };
+  auto smem_for = [&](int sg) { return (2 * 64 * sg * static_cast<int64_t>(g.cspan) + 64 * sg * 32 + nc) * 4; };
   if (p.tree_round == 64)
     g.sgroups = 1;
   else if (p.tree_round == 128)
-    g.sgroups = nchan % 128 == 0 ? 2 : 1;
+    g.sgroups = nc % 128 == 0 ? 2 : 1;
   else
-    g.sgroups = (nchan % 128 == 0 && smem_for(2) <= 100 * 1024) ? 2 : 1;
+    g.sgroups = (nc % 128 == 0 && smem_for(2) <= 100 * 1024) ? 2 : 1;
   const int64_t smem = smem_for(g.sgroups);
   if (smem > 200 * 1024) return;
   g.smem_bytes = static_cast<int>(smem);
-  p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nchan * 32, 0);
+  p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nc * 32, 0);
   for (int t = 0; t < g.ndm_tiles; ++t)
     for (int c = 0; c < nchan; ++c) {
-      const int32_t b4 = p.dbase[static_cast<size_t>(t) * nchan + c];
+      const int32_t b4 = p.dbase[static_cast<size_t>(t) * nc + c];
       for (int l = 0; l < 32; ++l) {
         const int d = std::min(ndm - 1, t * 32 + l);
         const int32_t v = p.delays[static_cast<size_t>(d) * nchan + c];
-        p.dmeta[(static_cast<size_t>(t) * nchan + c) * 32 + l] =
+        p.dmeta[(static_cast<size_t>(t) * nc + c) * 32 + l] =
             static_cast<uint16_t>((((v >> 5) - b4) << 5) | (v & 31));
       }
     }
   g.inst = inst;
+  g.nchan = nc;
   p.direct = true;
 }
 

@@ -83,6 +83,8 @@ enum {
 // Direct tree kernel geometry: CTA = 32 consecutive trial DMs (lane = DM) x warps * kw words.
 struct DirectGeom {
   int inst = kDirNone;
+  int nchan = 0;         // channels rounded up to a multiple of 64 (the rest are zero ring rows)
+  bool whole = true;     // every exact-level node (all modes: the channel count) is whole 64-channel groups
   int warps = 8;
   int kw = 4;
   int tile_words = 32;   // warps * kw
@@ -91,7 +93,7 @@ struct DirectGeom {
   int sgroups = 1;       // 64-channel adder groups staged per round (1 or 2)
   int smem_bytes = 0;
   int sub_lev = 0;       // graded: the exact level (first level whose nodes may exceed N)
-  int sub_groups = 1;    // graded: 64-channel groups per exact-level node
+  int sub_groups = 1;    // graded: 64-channel groups per exact-level node (the last may have fewer)
   int rates_inst = kDirNone;  // float / graded with per-level fire counts: the binary counting pass
   int rates_kw = 4;
 };

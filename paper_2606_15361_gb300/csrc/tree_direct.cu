@@ -44,7 +44,7 @@ constexpr long long kDirWaitCycles = kStageWaitCycles;
 
 struct DirArgs {
   const uint32_t* ring;
-  int R, nchan, ndm;
+  int R, nchan, ndm;       // nchan: a multiple of kDG (the channels past the plan's last stay zero)
   int B, KL, KI, N, nlev;
   int level_nodes[kMaxLevels];
   int sub_groups;          // graded: staged groups per exact-level node
@@ -256,7 +256,7 @@ struct DState<kGraded, KW, NPL, MAXU> {
   template <typename F>
   __device__ __forceinline__ void group(const DirArgs& a, int g, F& fetch) {
     add_group<KW, NPL>(P, fetch);
-    if ((g + 1) % a.sub_groups != 0) return;
+    if ((g + 1) % a.sub_groups != 0 && g + 1 != a.nchan / kDG) return;
     // an exact-level node is complete: its value min(count, N) goes up the capped levels
     uint32_t cur[KW][8];
 #pragma unroll
@@ -382,9 +382,11 @@ struct DState<kBinary, KW, NPL, MAXU> {
   }
   // the 16 leaves of a staged group, each the quorum >= KL of its four channel bits
   template <int KL, typename F>
-  __device__ __forceinline__ void leaves(const DirArgs& a, F& fetch) {
+  __device__ __forceinline__ void leaves(const DirArgs& a, int g, F& fetch) {
+    const int nleaf = a.level_nodes[0] - g * (kDG / 4);  // leaves from this group on
 #pragma unroll 4
     for (int k = 0; k < kDG / 4; ++k) {
+      if (k >= nleaf) break;  // leaves of the channels past the last are not part of the tree
       uint32_t x0[KW], x1[KW], x2[KW], x3[KW], v[KW];
       fetch(4 * k, x0);
       fetch(4 * k + 1, x1);
@@ -410,12 +412,12 @@ struct DState<kBinary, KW, NPL, MAXU> {
     }
   }
   template <typename F>
-  __device__ __forceinline__ void group(const DirArgs& a, int, F& fetch) {
+  __device__ __forceinline__ void group(const DirArgs& a, int g, F& fetch) {
     switch (a.KL) {
-      case 1: leaves<1>(a, fetch); break;
-      case 2: leaves<2>(a, fetch); break;
-      case 3: leaves<3>(a, fetch); break;
-      default: leaves<4>(a, fetch); break;
+      case 1: leaves<1>(a, g, fetch); break;
+      case 2: leaves<2>(a, g, fetch); break;
+      case 3: leaves<3>(a, g, fetch); break;
+      default: leaves<4>(a, g, fetch); break;
     }
   }
   __device__ __forceinline__ void store(int32_t* row, int j) const { store_bits(row, root[j]); }
@@ -543,20 +545,24 @@ struct DState {
       }
     }
   }
+  // left: level-UIN nodes from this group on. Channels past the last never fire, so they change no
+  // node that has real ones; a node of nothing else is not part of the tree.
   template <int KL, int K, typename F>
-  __device__ __forceinline__ void tops(const DirArgs& a, F& fetch) {
+  __device__ __forceinline__ void tops(const DirArgs& a, int left, F& fetch) {
+    if (K >= left) return;
     uint32_t v[KW];
     node<KL, UIN, K * SPAN>(fetch, v);
     push(a, v);
-    if constexpr (K + 1 < NTOP) tops<KL, K + 1>(a, fetch);
+    if constexpr (K + 1 < NTOP) tops<KL, K + 1>(a, left, fetch);
   }
   template <typename F>
-  __device__ __forceinline__ void group(const DirArgs& a, int, F& fetch) {
+  __device__ __forceinline__ void group(const DirArgs& a, int g, F& fetch) {
+    const int left = a.level_nodes[UIN] - g * NTOP;
     switch (a.KL) {
-      case 1: tops<1, 0>(a, fetch); break;
-      case 2: tops<2, 0>(a, fetch); break;
-      case 3: tops<3, 0>(a, fetch); break;
-      default: tops<4, 0>(a, fetch); break;
+      case 1: tops<1, 0>(a, left, fetch); break;
+      case 2: tops<2, 0>(a, left, fetch); break;
+      case 3: tops<3, 0>(a, left, fetch); break;
+      default: tops<4, 0>(a, left, fetch); break;
     }
   }
   __device__ __forceinline__ void store(int32_t* row, int j) const { store_bits(row, root[j]); }
@@ -791,7 +797,7 @@ void direct_args(const Plan& p, int64_t e_prev, int64_t e_new, DirArgs& a, int* 
   a = DirArgs{};
   a.ring = dp.ring;
   a.R = p.R;
-  a.nchan = p.nchan;
+  a.nchan = g.nchan;
   a.ndm = p.ndm;
   a.B = p.B;
   a.KL = p.KL;
