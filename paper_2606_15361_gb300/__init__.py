@@ -277,13 +277,12 @@ class Plan:
     def candidates(self, cap: int | None = None, check: bool = True):
         """Synchronise and return (structured numpy array of candidates, status)."""
         cap = int(self.opts.cand_capacity if cap is None else cap)
-        buf = (SndCandidate * max(cap, 1))()
+        buf = np.empty(max(cap, 1), dtype=CANDIDATE_DTYPE)  # pages are touched only where a candidate lands
         n = ctypes.c_int32(0)
-        rc = lib.snd_candidates(self.handle, buf, cap, ctypes.byref(n))
+        rc = lib.snd_candidates(self.handle, buf.ctypes.data_as(ctypes.POINTER(SndCandidate)), cap, ctypes.byref(n))
         if check:
             _check(rc, "snd_candidates")
-        arr = np.frombuffer(bytes(buf)[: n.value * CANDIDATE_DTYPE.itemsize], dtype=CANDIDATE_DTYPE).copy()
-        return arr, rc
+        return buf[: n.value].copy(), rc
 
     def stats(self) -> SndPlanStats:
         s = SndPlanStats()
@@ -404,13 +403,12 @@ class MultiRatePlan:
     def candidates(self, cap: int | None = None, check: bool = True):
         """Merged candidates since the last call: (structured numpy array, status)."""
         cap = int(self.opts.cand_capacity * len(self.scrunch) if cap is None else cap)
-        buf = (SndCandidate * max(cap, 1))()
+        buf = np.empty(max(cap, 1), dtype=CANDIDATE_DTYPE)  # pages are touched only where a candidate lands
         n = ctypes.c_int32(0)
-        rc = lib.snd_multirate_candidates(self.handle, buf, cap, ctypes.byref(n))
+        rc = lib.snd_multirate_candidates(self.handle, buf.ctypes.data_as(ctypes.POINTER(SndCandidate)), cap, ctypes.byref(n))
         if check:
             _check(rc, "snd_multirate_candidates")
-        arr = np.frombuffer(bytes(buf)[: n.value * CANDIDATE_DTYPE.itemsize], dtype=CANDIDATE_DTYPE).copy()
-        return arr, rc
+        return buf[: n.value].copy(), rc
 
 
 def _ptr(t):

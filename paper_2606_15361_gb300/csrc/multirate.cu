@@ -47,6 +47,7 @@ struct MultiRate {
   snd::GraphRunner runner;
   cudaStream_t last_stream = nullptr;
   int sticky = 0;
+  snd::HostRead read;  // snd_multirate_candidates
 };
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -447,14 +448,18 @@ extern "C" int snd_multirate_candidates(snd_multirate_t h, snd_candidate_t* host
   k_best<<<64, 256, 0, s>>>(all, cnt, m.cap, parent, best, tie, 1);
   k_emit_sorted<<<64, 256, 0, s>>>(all, cnt, m.cap, parent, best, tie, outd, cnt + 1);
   if (cudaGetLastError() != cudaSuccess) return fail(m, SND_ERR_CUDA);
-  uint32_t hc[4];
-  if (cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  if (!m.read.ready()) return fail(m, SND_ERR_NOMEM);
+  const uint32_t* hc = m.read.counters;
+  const int head = static_cast<int>(std::min<int64_t>(std::min<int64_t>(cap, m.cap), snd::kReadCands));
+  if (cudaMemcpyAsync(m.read.counters, cnt, sizeof(uint32_t) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      (head > 0 && cudaMemcpyAsync(m.read.cand, outd, sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
+                       cudaSuccess) ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return fail(m, SND_ERR_CUDA);
   const int n = static_cast<int>(hc[1]);
   const int take = std::min(n, cap);
-  if (take > 0 && cudaMemcpy(host_out, outd, sizeof(snd_candidate_t) * take, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return fail(m, SND_ERR_CUDA);
+  if (take > 0) std::memcpy(host_out, m.read.cand, sizeof(snd_candidate_t) * std::min(take, head));
+  if (snd::read_tail(outd, take, host_out, s) != cudaSuccess) return fail(m, SND_ERR_CUDA);
   *n_out = take;
   const uint32_t st = hc[2] | hc[3];
   if (st & (snd::kStatusTauTimeout | snd::kStatusUnionTimeout)) return SND_ERR_TIMEOUT;

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include "snd_internal.h"
@@ -32,6 +33,36 @@ void chunk_commit(Plan& p, const ChunkPos& c, int32_t nsamp, cudaStream_t s) {
   p.F = (p.mode == SND_MODE_ZFLOAT) ? p.F : c.f_new;
   p.last_stream = s;
   p.pending_host = -1;
+}
+
+bool HostRead::ready() {
+  if (counters) return true;
+  constexpr size_t head = 64, bytes = head + sizeof(snd_candidate_t) * kReadCands;
+  static_assert(sizeof(uint32_t) * kCntSlots <= head, "counters before the candidates");
+  void* m = nullptr;
+  if (cudaHostAlloc(&m, bytes, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    try {
+      pageable.resize(bytes + alignof(snd_candidate_t));
+    } catch (const std::bad_alloc&) {
+      return false;
+    }
+    m = pageable.data();
+  }
+  counters = static_cast<uint32_t*>(m);
+  cand = reinterpret_cast<snd_candidate_t*>(static_cast<unsigned char*>(m) + head);
+  return true;
+}
+
+HostRead::~HostRead() {
+  if (counters && pageable.empty()) cudaFreeHost(counters);
+}
+
+cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s) {
+  if (take <= kReadCands) return cudaSuccess;
+  const cudaError_t e = cudaMemcpyAsync(host_out + kReadCands, src + kReadCands,
+                                        sizeof(snd_candidate_t) * (take - kReadCands), cudaMemcpyDeviceToHost, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
 }  // namespace snd
@@ -321,18 +352,23 @@ extern "C" int snd_candidates(snd_plan_t plan, snd_candidate_t* host_out, int32_
   Plan& p = *reinterpret_cast<Plan*>(plan);
   if (!p.bound) return SND_ERR_STATE;
   if (p.sticky) return p.sticky;
-  if (cudaStreamSynchronize(p.last_stream) != cudaSuccess) return fail(p, SND_ERR_CUDA);
-  uint32_t cnt[snd::kCntSlots];
-  if (cudaMemcpy(cnt, p.dp.counters, sizeof(cnt), cudaMemcpyDeviceToHost) != cudaSuccess)
+  // the counters, the head of the list and the reset of its count and status word (adjacent) in the
+  // stream's order, one wait for all three
+  if (!p.read.ready()) return fail(p, SND_ERR_NOMEM);
+  cudaStream_t s = p.last_stream;
+  const uint32_t* cnt = p.read.counters;
+  const int head = std::min(std::min(cap, p.cand_cap), snd::kReadCands);
+  if (cudaMemcpyAsync(p.read.counters, p.dp.counters, sizeof(uint32_t) * snd::kCntSlots, cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      (head > 0 && cudaMemcpyAsync(p.read.cand, p.dp.cand, sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
+                       cudaSuccess) ||
+      cudaMemsetAsync(p.dp.counters + snd::kCntCands, 0, sizeof(uint32_t) * 2, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
     return fail(p, SND_ERR_CUDA);
   const int n = static_cast<int>(cnt[snd::kCntCands]);
   const int take = n < cap ? n : cap;
-  if (take > 0 &&
-      cudaMemcpy(host_out, p.dp.cand, sizeof(snd_candidate_t) * take, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return fail(p, SND_ERR_CUDA);
-  uint32_t zero[2] = {0, 0};
-  if (cudaMemcpy(p.dp.counters + snd::kCntCands, zero, sizeof(zero), cudaMemcpyHostToDevice) != cudaSuccess)
-    return fail(p, SND_ERR_CUDA);
+  if (take > 0) std::memcpy(host_out, p.read.cand, sizeof(snd_candidate_t) * std::min(take, head));
+  if (snd::read_tail(p.dp.cand, take, host_out, s) != cudaSuccess) return fail(p, SND_ERR_CUDA);
   *n_out = take;
   p.pending_host = 0;
   const uint32_t st = cnt[snd::kCntStatus];

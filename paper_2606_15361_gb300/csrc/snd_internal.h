@@ -187,6 +187,20 @@ enum {
   kCntSlots = 16
 };
 
+// Where a plan's counters and the head of its candidate list are read back to: page-locked, so both
+// copies and the reset of the list wait on the GPU once. Allocated at the first read, freed with its
+// owner. Candidate lists past kReadCands take a second copy.
+constexpr int kReadCands = 512;
+struct HostRead {
+  uint32_t* counters = nullptr;      // [kCntSlots]
+  snd_candidate_t* cand = nullptr;   // [kReadCands]
+  std::vector<unsigned char> pageable;  // in use when page-locked memory is not to be had
+  bool ready();
+  ~HostRead();
+};
+// Head of the list: the n candidates at `src` (device) from kReadCands on go to host_out directly.
+cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s);
+
 struct Plan {
   // configuration
   int nchan = 0, ndm = 0, mode = 0, B = 2, C = 4, KL = 2, KI = 2, N = 255;
@@ -261,6 +275,8 @@ struct Plan {
   cudaEvent_t up_free[2] = {nullptr, nullptr};  // the chunk that read buffer b finished
   bool up_free_set[2] = {false, false};
   int up_next = 0;
+
+  HostRead read;  // snd_candidates
 
   // per-stage timing (snd_profile)
   bool profiling = false;
