@@ -8,11 +8,17 @@
 //   S1c = (S1in + n_lo lo) + n_hi hi, S2c = (S2in + n_lo lo^2) + n_hi hi^2,
 //   mu = S1c/n, sigma = sqrt(max(0, S2c/n - mu^2)), u = min{v in 0..255 : v > mu + theta sigma}.
 //
+// Two forms: k_encode does a whole chunk of a block of 32 channels in one launch, with a cluster's
+// CTAs holding the samples in shared memory between the statistics and the packing; the labelled
+// payload, and chunks too long for that, take k_hist, k_levels and a pack kernel.
+//
 // Ring layout: ring[c][2R] uint32; absolute sample a lives in word a>>5, bit a&31, stored at
 // physical word (a>>5) mod R and again at R + that (the mirror lets any window of < R words
 // be read contiguously).
 
 #include <cuda_fp16.h>
+
+#include <algorithm>
 
 #include "snd_internal.h"
 
@@ -259,74 +265,376 @@ __global__ void __launch_bounds__(256) k_pack32(const uint8_t* __restrict__ chun
               threadIdx.x & 31);
 }
 
-// Many plans' encoders, three launches in all: every kernel's CTAs are spread over the beams
-// by a prefix of their CTA counts (a CTA finds its beam by binary search).
-constexpr int kMaxEncBeams = 64;
-
+// One beam's chunk for k_encode. A cluster of S CTAs takes 32 channels; CTA `rank` of it the ring words
+// w0 + rank * wpc .. (wpc words), i.e. those words' samples.
 struct EncBeam {
   const uint8_t* chunk;
   int nsamp, nchan;
-  uint32_t* hist;
   int32_t* levels;
   double theta;
   long long t0, w0;
-  int nwords;
+  int nwords, wpc;
   uint32_t* ring;
   int R;
+  int vec;             // bytes per load: 16, 4 or 1 (what the chunk's address and nchan allow)
   uint32_t* counters;  // the beam's matched-filter / candidate block counters, cleared here
-  int hx;              // histogram CTAs along channels
 };
+
+constexpr int kMaxEncBeams = 64;
+constexpr int kEncCluster = 8;  // most CTAs of a cluster
+// A CTA of 256 threads where four fit an SM's shared memory, of 512 where fewer do.
+constexpr int kEncSmall = 54 * 1024;
 
 struct EncMulti {
   int nbeams;
-  int first_h[kMaxEncBeams], first_l[kMaxEncBeams], first_p[kMaxEncBeams];
+  int first[kMaxEncBeams];  // clusters of the beams before
   EncBeam beam[kMaxEncBeams];
 };
 
-__device__ __forceinline__ int beam_of(const int* first, int n, int i) {
-  int lo = 0, hi = n - 1;
+// shared memory of a CTA: the samples and the packed words
+__host__ __device__ constexpr int enc_smem(int wpc) { return wpc * 32 * 32 + 32 * (wpc | 1) * 4; }
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v into the 32-bit word at shared address `addr` of every CTA of the cluster (visible after the next
+// cluster barrier): pushed rather than read later, so no load waits on another SM
+__device__ __forceinline__ void cluster_put(uint32_t addr, uint32_t v, int S) {
+  for (int r = 0; r < S; ++r) {
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(r));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(v) : "memory");
+  }
+}
+
+// Encoder of one chunk in one launch. What bounded the three-kernel form was latency, not bytes: three
+// dependent launches, global atomics between them, and a second read of the chunk in 4-byte ring
+// stores. Here each CTA brings its samples into shared memory once (asynchronous copies, all in flight
+// together) and sums them per channel, the cluster adds its CTAs' sums through distributed shared
+// memory, one warp evaluates the FP64 recipe for all 32 channels at once (lane = channel), a second
+// pass over the shared samples sums what the clip bounds leave out, and the same samples are compared
+// and packed; ring words leave as contiguous runs per channel. No histogram: with the samples in
+// shared memory two passes of exact integer sums cost less than its atomics (with them 24 us for 64
+// channels, 56 us for 1024). Sums and FP64 steps are those of levels_warp, so the levels are the same.
+// Encoder stage (with its event pair): 1024 channels x 16384 samples 48 -> 27 us, 4096 x 7246 80 -> 41,
+// 1000 x 10007 54 -> 29 (4-byte loads), 64 x 1024 26 -> 16.
+template <int kEncThreads>
+__device__ __forceinline__ void encode_cta(const EncBeam& e, const int cb, unsigned char* sm) {
+  constexpr int NW = kEncThreads / 32;
+  __shared__ uint32_t red[NW][4][32];
+  // every CTA's totals: sum and sum of squares; count below, count above, sum and sum of squares of both
+  __shared__ uint32_t tot1[kEncCluster][2][32], tot2[kEncCluster][4][32];
+  __shared__ int clip[2][32], lev[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int rank = static_cast<int>(cluster_rank()), S = static_cast<int>(cluster_size());
+  unsigned char* tile = sm;                                // [wpc * 32][32]
+  uint32_t* bits = reinterpret_cast<uint32_t*>(tile + e.wpc * 32 * 32);  // [32][wpc | 1]
+  const int c0 = cb * 32;
+  const int q0 = rank * e.wpc, nq = max(0, min(e.wpc, e.nwords - q0));  // this CTA's ring words
+  const long long aw0 = e.w0 + q0;
+  const int rbase = static_cast<int>(aw0 * 32 - e.t0);     // chunk row of tile row 0 (negative in the first word)
+  const int i0 = max(0, -rbase), i1 = min(nq * 32, e.nsamp - rbase);  // tile rows that are in the chunk
+
+  // the samples of [i0, i1) x 32 channels (bytes past the last channel stay unread)
+  const uint8_t* src = e.chunk + static_cast<long long>(rbase) * e.nchan + c0;
+  const int nc = min(32, e.nchan - c0);
+  const uint32_t stile = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
+  if (e.vec == 16) {
+    const int per = nc >> 4;  // 16-byte pieces a row
+    for (int i = i0 * 2 + tid; i < i1 * 2; i += kEncThreads) {
+      const int row = i >> 1, p = i & 1;
+      if (p < per)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stile + row * 32 + p * 16),
+                     "l"(src + static_cast<long long>(row) * e.nchan + p * 16)
+                     : "memory");
+    }
+  } else if (e.vec == 4) {
+    const int per = nc >> 2;
+    for (int i = i0 * 8 + tid; i < i1 * 8; i += kEncThreads) {
+      const int row = i >> 3, p = i & 7;
+      if (p < per)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(stile + row * 32 + p * 4),
+                     "l"(src + static_cast<long long>(row) * e.nchan + p * 4)
+                     : "memory");
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  if (e.vec == 1 && lane < nc) {
+    int i = i0 + wid;
+    for (; i + 7 * NW < i1; i += 8 * NW) {
+      uint8_t v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = __ldg(src + static_cast<long long>(i + NW * k) * e.nchan + lane);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) tile[(i + NW * k) * 32 + lane] = v[k];
+    }
+    for (; i < i1; i += NW) tile[i * 32 + lane] = __ldg(src + static_cast<long long>(i) * e.nchan + lane);
+  }
+  cluster_arrive();  // the peers' shared memory may be written once they have all started
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+
+  // first pass: sums over the chunk, lane = channel (a CTA's fit 32 bits: at most 6.6e4 samples of
+  // 255^2; channels past the last sum what was there, and are not written out)
+  uint32_t a1 = 0, a2 = 0;
+  {
+    int i = i0 + wid;
+    for (; i + 7 * NW < i1; i += 8 * NW) {
+      uint32_t v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = tile[(i + NW * k) * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        a1 += v[k];
+        a2 += v[k] * v[k];
+      }
+    }
+    for (; i < i1; i += NW) {
+      const uint32_t v = tile[i * 32 + lane];
+      a1 += v;
+      a2 += v * v;
+    }
+  }
+  red[wid][0][lane] = a1;
+  red[wid][1][lane] = a2;
+  cluster_wait();
+  __syncthreads();
+  if (wid < 2) {
+    uint32_t s = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) s += red[w][wid][lane];
+    cluster_put(static_cast<uint32_t>(__cvta_generic_to_shared(&tot1[rank][wid][lane])), s, S);
+  }
+  cluster_arrive();
+  cluster_wait();
+  const double nf = static_cast<double>(e.nsamp);
+  double lo = 0.0, hi = 0.0;
+  long long s1 = 0, s2 = 0;  // of the chunk, in warp 0
+  if (wid == 0) {
+    for (int r = 0; r < S; ++r) {
+      s1 += tot1[r][0][lane];
+      s2 += tot1[r][1][lane];
+    }
+    const double mu0 = __ddiv_rn(static_cast<double>(s1), nf);
+    const double var0 = __dsub_rn(__ddiv_rn(static_cast<double>(s2), nf), __dmul_rn(mu0, mu0));
+    const double sig0 = var0 > 0.0 ? __dsqrt_rn(var0) : 0.0;
+    lo = __dsub_rn(mu0, __dmul_rn(5.0, sig0));
+    hi = __dadd_rn(mu0, __dmul_rn(5.0, sig0));
+    clip[0][lane] = static_cast<int>(fmin(fmax(ceil(lo), -1.0), 257.0));
+    clip[1][lane] = static_cast<int>(fmin(fmax(floor(hi), -1.0), 257.0));
+  }
+  __syncthreads();
+  // second pass: the values outside the clip bounds: how many below and above, and their sums. They
+  // are few (5 sigma), so eight rows are tested at once and a warp only goes through them one by one
+  // where a lane has one (testing and adding row by row took 17,000 cycles of 2,080 rows, this an eighth)
+  {
+    const int ilo = clip[0][lane], ihi = clip[1][lane];
+    uint32_t s1 = 0, s2 = 0, nlo = 0, nhi = 0;
+    auto out = [&](int v) {
+      if (v < ilo) ++nlo; else if (v > ihi) ++nhi; else return;
+      s1 += v;
+      s2 += v * v;
+    };
+    int i = i0 + wid;
+    for (; i + 7 * NW < i1; i += 8 * NW) {
+      int v[8], least = 255, most = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = tile[(i + NW * k) * 32 + lane];
+        least = min(least, v[k]);
+        most = max(most, v[k]);
+      }
+      if (__any_sync(0xFFFFFFFFu, lane < nc && (least < ilo || most > ihi))) {
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) out(tile[(i + NW * k) * 32 + lane]);
+      }
+    }
+    for (; i < i1; i += NW) out(tile[i * 32 + lane]);
+    red[wid][0][lane] = nlo;
+    red[wid][1][lane] = nhi;
+    red[wid][2][lane] = s1;
+    red[wid][3][lane] = s2;
+  }
+  __syncthreads();
+  if (wid < 4) {
+    uint32_t s = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) s += red[w][wid][lane];
+    cluster_put(static_cast<uint32_t>(__cvta_generic_to_shared(&tot2[rank][wid][lane])), s, S);
+  }
+  cluster_arrive();
+  cluster_wait();
+  if (wid == 0) {
+    long long nlo = 0, nhi = 0, s1in = s1, s2in = s2;
+    for (int r = 0; r < S; ++r) {
+      nlo += tot2[r][0][lane];
+      nhi += tot2[r][1][lane];
+      s1in -= tot2[r][2][lane];
+      s2in -= tot2[r][3][lane];
+    }
+    const double s1c = __dadd_rn(__dadd_rn(static_cast<double>(s1in), __dmul_rn(static_cast<double>(nlo), lo)),
+                                 __dmul_rn(static_cast<double>(nhi), hi));
+    const double s2c =
+        __dadd_rn(__dadd_rn(static_cast<double>(s2in), __dmul_rn(static_cast<double>(nlo), __dmul_rn(lo, lo))),
+                  __dmul_rn(static_cast<double>(nhi), __dmul_rn(hi, hi)));
+    const double mu = __ddiv_rn(s1c, nf);
+    const double var = __dsub_rn(__ddiv_rn(s2c, nf), __dmul_rn(mu, mu));
+    const double sig = var > 0.0 ? __dsqrt_rn(var) : 0.0;
+    int u = 256;
+    if (sig > 0.0) {
+      const double thr = __dadd_rn(mu, __dmul_rn(e.theta, sig));
+      if (thr < 0.0) {
+        u = 0;
+      } else if (thr < 255.0) {
+        u = static_cast<int>(floor(thr)) + 1;
+      }
+    }
+    lev[lane] = u;
+    if (rank == 0 && lane < nc) e.levels[c0 + lane] = u;
+  }
+  __syncthreads();
+
+  // pack: a warp per ring word, lane = sample. P >= u for four channels at a time: v + (256 - u) in
+  // 16-bit halves carries into bit 8 exactly when it holds (u <= 256); the lane's 32 bits are gathered
+  // byte by byte (bit 8 b + i = channel 4 i + b) and a 32 x 32 transpose over the warp turns samples'
+  // words into channels' (a ballot per channel took four times as long).
+  const int bp = e.wpc | 1;  // odd pitch: the lanes' words fall into different banks
+  uint32_t ke[8], ko[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    ke[i] = static_cast<uint32_t>(256 - lev[4 * i]) | (static_cast<uint32_t>(256 - lev[4 * i + 2]) << 16);
+    ko[i] = static_cast<uint32_t>(256 - lev[4 * i + 1]) | (static_cast<uint32_t>(256 - lev[4 * i + 3]) << 16);
+  }
+  for (int q = wid; q < nq; q += NW) {
+    const int i = q * 32 + lane;
+    const uint4 b0 = *reinterpret_cast<const uint4*>(tile + i * 32), b1 = *reinterpret_cast<const uint4*>(tile + i * 32 + 16);
+    const uint32_t wv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+    uint32_t x = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t ev = (wv[j] & 0x00FF00FFu) + ke[j], od = ((wv[j] >> 8) & 0x00FF00FFu) + ko[j];
+      x += __byte_perm(ev, od, 0x7351) << j;  // bytes 1 and 3 of both: 0 or 1 each
+    }
+    if (i < i0 || i >= i1) x = 0;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+      const uint32_t m = j == 16 ? 0x0000FFFFu : (j == 8 ? 0x00FF00FFu : (j == 4 ? 0x0F0F0F0Fu : (j == 2 ? 0x33333333u : 0x55555555u)));
+      const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
+      x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
+    }
+    bits[(4 * (lane & 7) + (lane >> 3)) * bp + q] = x;
+  }
+  __syncthreads();
+  const int phys0 = static_cast<int>(aw0 % e.R);
+  for (int c = wid; c < nc; c += NW) {
+    uint32_t* row = e.ring + static_cast<size_t>(c0 + c) * 2 * e.R;
+    for (int q = lane; q < nq; q += 32) {
+      int phys = phys0 + q;
+      if (phys >= e.R) phys -= e.R;
+      uint32_t w = bits[c * bp + q];
+      // only the chunk's first word keeps bits of samples before the chunk (previous chunk)
+      if (rank == 0 && q == 0 && rbase < 0) w |= row[phys] & ((1u << -rbase) - 1u);
+      row[phys] = w;
+      row[phys + e.R] = w;
+    }
+  }
+}
+
+__device__ __forceinline__ void clear_block_counters(const EncBeam& e) {
+  e.counters[kCntCells] = 0;
+  e.counters[kCntRuns] = 0;
+  e.counters[kCntBlockCands] = 0;
+}
+
+// one plan: cluster i takes channels 32 i ..
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_encode(const __grid_constant__ EncBeam e) {
+  extern __shared__ __align__(16) unsigned char esm[];
+  if (blockIdx.x == 0 && threadIdx.x == 0) clear_block_counters(e);
+  encode_cta<NT>(e, static_cast<int>(blockIdx.x) / static_cast<int>(cluster_size()), esm);
+}
+
+// many plans: cluster i takes channels 32 (i - first[b]) .. of the last beam b with first[b] <= i
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_encode_multi(const __grid_constant__ EncMulti m) {
+  extern __shared__ __align__(16) unsigned char esm[];
+  const int i = static_cast<int>(blockIdx.x) / static_cast<int>(cluster_size());
+  int lo = 0, hi = m.nbeams - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (first[mid] <= i) lo = mid; else hi = mid - 1;
+    if (m.first[mid] <= i) lo = mid; else hi = mid - 1;
   }
-  return lo;
+  const EncBeam& e = m.beam[lo];
+  if (i == m.first[lo] && cluster_rank() == 0 && threadIdx.x == 0) clear_block_counters(e);
+  encode_cta<NT>(e, i - m.first[lo], esm);
 }
 
-__global__ void __launch_bounds__(32 * kHistWarps) k_hist_multi(const __grid_constant__ EncMulti m) {
-  const int i = static_cast<int>(blockIdx.x);
-  const int b = beam_of(m.first_h, m.nbeams, i);
-  const EncBeam& e = m.beam[b];
-  const int local = i - m.first_h[b];
-  hist_cta(e.chunk, e.nsamp, e.nchan, e.hist, local % e.hx, local / e.hx);
+// Whether k_encode takes this plan's chunk at S CTAs per cluster; fills e.
+bool enc_beam(const Plan& p, const uint8_t* chunk, int nsamp, int S, EncBeam& e) {
+  if (p.mode == SND_MODE_ZFLOAT) return false;
+  e.chunk = chunk;
+  e.nsamp = nsamp;
+  e.nchan = p.nchan;
+  e.levels = p.dp.levels;
+  e.theta = p.enc_theta;
+  e.t0 = p.T;
+  e.w0 = p.T >> 5;
+  e.nwords = static_cast<int>(((p.T + nsamp - 1) >> 5) - e.w0 + 1);
+  e.wpc = (e.nwords + S - 1) / S;
+  e.ring = p.dp.ring;
+  e.R = p.R;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(chunk) | static_cast<uintptr_t>(p.nchan);
+  e.vec = (at & 15u) == 0 ? 16 : ((at & 3u) == 0 ? 4 : 1);
+  e.counters = p.dp.counters;
+  return enc_smem(e.wpc) <= 220 * 1024 && e.nwords <= e.R;
 }
 
-__global__ void __launch_bounds__(256) k_levels_multi(const __grid_constant__ EncMulti m) {
-  const int i = static_cast<int>(blockIdx.x);
-  const int b = beam_of(m.first_l, m.nbeams, i);
-  const EncBeam& e = m.beam[b];
-  const int local = i - m.first_l[b];
-  if (local == 0 && threadIdx.x == 0) {
-    e.counters[kCntCells] = 0;
-    e.counters[kCntRuns] = 0;
-    e.counters[kCntBlockCands] = 0;
-  }
-  levels_warp(e.hist, e.nchan, e.nsamp, e.theta, e.levels, nullptr, 0, local * 8 + (threadIdx.x >> 5),
-              threadIdx.x & 31);
-}
-
-__global__ void __launch_bounds__(256) k_pack32_multi(const __grid_constant__ EncMulti m) {
-  const int i = static_cast<int>(blockIdx.x);
-  const int b = beam_of(m.first_p, m.nbeams, i);
-  const EncBeam& e = m.beam[b];
-  const int local = i - m.first_p[b];
-  pack32_warp(e.chunk, e.nsamp, e.nchan, e.levels, e.t0, e.w0, e.nwords, e.ring, e.R,
-              local * 8 + (threadIdx.x >> 5), threadIdx.x & 31);
+template <typename A>
+cudaError_t run_encode(void (*kern)(A), int threads, const A& args, int clusters, int S, int smem, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(clusters) * S);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = S;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args);
 }
 
 }  // namespace
 
 cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cudaStream_t s) {
   const DevPtrs& dp = p.dp;
+  {
+    // eight CTAs a cluster, fewer for chunks of few words (at least eight words each)
+    const int nwords = static_cast<int>(((p.T + nsamp - 1) >> 5) - (p.T >> 5) + 1);
+    int S = kEncCluster;
+    while (S > 1 && nwords < 8 * S) S /= 2;
+    EncBeam b{};
+    if (enc_beam(p, d_chunk, nsamp, S, b)) {
+      p.launches += 1;
+      const int smem = enc_smem(b.wpc), clusters = (p.nchan + 31) / 32;
+      return smem <= kEncSmall ? run_encode(k_encode<256>, 256, b, clusters, S, smem, s)
+                               : run_encode(k_encode<512>, 512, b, clusters, S, smem, s);
+    }
+  }
+  cudaError_t ec = cudaMemsetAsync(dp.counters, 0, sizeof(uint32_t) * (kCntBlockCands + 1), s);
+  if (ec != cudaSuccess) return ec;
   dim3 hb(32, kHistWarps), hg((p.nchan + 31) / 32, (nsamp + kHistRowsPerBlock - 1) / kHistRowsPerBlock);
   k_hist<<<hg, hb, 0, s>>>(d_chunk, nsamp, p.nchan, dp.hist);
   const bool z = p.mode == SND_MODE_ZFLOAT;
@@ -360,63 +668,51 @@ cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cuda
   return cudaGetLastError();
 }
 
-// Encoders of several plans (bit-ring modes, 32-channel multiples, 16-byte aligned chunks) in
-// three launches; each beam's matched-filter and candidate block counters are cleared by its
-// first levels CTA. Plans outside those conditions take their own launch_encode (and the
-// counters are cleared by a memset).
+// Encoders of several plans in one launch per shared-memory class (54 KB a CTA: four fit an SM;
+// 110 KB: two; more: one), so a long-chunk beam does not lower every other beam's occupancy; more
+// launches only past kMaxEncBeams beams of a class. Plans that k_encode does not take run their own
+// launch_encode.
 cudaError_t launch_encode_batch(const Plan* const* plans, const uint8_t* const* chunks, const int32_t* nsamp, int n,
                                 cudaStream_t s) {
+  constexpr int S = kEncCluster;
+  auto cls = [](int smem) { return smem <= kEncSmall ? 0 : (smem <= 110 * 1024 ? 1 : 2); };
   EncMulti m{};
-  int nh = 0, nl = 0, np = 0;
+  int clusters = 0, smem = 0;
   const Plan* owner = nullptr;
-  auto flush = [&]() -> cudaError_t {
+  auto flush = [&](int c) -> cudaError_t {
     if (m.nbeams == 0) return cudaSuccess;
-    k_hist_multi<<<nh, dim3(32, kHistWarps), 0, s>>>(m);
-    k_levels_multi<<<nl, 256, 0, s>>>(m);
-    k_pack32_multi<<<np, 256, 0, s>>>(m);
-    owner->launches += 3;
+    const cudaError_t e = c == 0 ? run_encode(k_encode_multi<256>, 256, m, clusters, S, smem, s)
+                                 : run_encode(k_encode_multi<512>, 512, m, clusters, S, smem, s);
+    owner->launches += 1;
     m.nbeams = 0;
-    nh = nl = np = 0;
+    clusters = smem = 0;
     owner = nullptr;
-    return cudaGetLastError();
+    return e;
   };
-  for (int i = 0; i < n; ++i) {
-    const Plan& p = *plans[i];
-    const bool fits = p.mode != SND_MODE_ZFLOAT && p.nchan % 32 == 0 &&
-                      (reinterpret_cast<uintptr_t>(chunks[i]) & 15u) == 0;
-    if (!fits) {
-      cudaError_t e = launch_encode(p, chunks[i], nsamp[i], s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(p.dp.counters, 0, sizeof(uint32_t) * (kCntBlockCands + 1), s);
-      if (e != cudaSuccess) return e;
-      continue;
+  for (int c = 0; c < 3; ++c) {
+    for (int i = 0; i < n; ++i) {
+      const Plan& p = *plans[i];
+      EncBeam& b = m.beam[m.nbeams];
+      if (!enc_beam(p, chunks[i], nsamp[i], S, b)) {
+        if (c != 0) continue;
+        const cudaError_t e = launch_encode(p, chunks[i], nsamp[i], s);
+        if (e != cudaSuccess) return e;
+        continue;
+      }
+      if (cls(enc_smem(b.wpc)) != c) continue;
+      m.first[m.nbeams] = clusters;
+      clusters += (p.nchan + 31) / 32;
+      smem = std::max(smem, enc_smem(b.wpc));
+      if (!owner) owner = &p;
+      if (++m.nbeams == kMaxEncBeams) {
+        const cudaError_t e = flush(c);
+        if (e != cudaSuccess) return e;
+      }
     }
-    EncBeam& e = m.beam[m.nbeams];
-    e.chunk = chunks[i];
-    e.nsamp = nsamp[i];
-    e.nchan = p.nchan;
-    e.hist = p.dp.hist;
-    e.levels = p.dp.levels;
-    e.theta = p.enc_theta;
-    e.t0 = p.T;
-    e.w0 = p.T >> 5;
-    e.nwords = static_cast<int>(((p.T + nsamp[i] - 1) >> 5) - e.w0 + 1);
-    e.ring = p.dp.ring;
-    e.R = p.R;
-    e.counters = p.dp.counters;
-    e.hx = (p.nchan + 31) / 32;
-    m.first_h[m.nbeams] = nh;
-    m.first_l[m.nbeams] = nl;
-    m.first_p[m.nbeams] = np;
-    nh += e.hx * ((nsamp[i] + kHistRowsPerBlock - 1) / kHistRowsPerBlock);
-    nl += (p.nchan * 32 + 255) / 256;
-    np += static_cast<int>((static_cast<long long>(e.nwords) * (p.nchan / 32) * 32 + 255) / 256);
-    if (!owner) owner = &p;
-    if (++m.nbeams == kMaxEncBeams) {
-      const cudaError_t err = flush();
-      if (err != cudaSuccess) return err;
-    }
+    const cudaError_t e = flush(c);
+    if (e != cudaSuccess) return e;
   }
-  return flush();
+  return cudaSuccess;
 }
 
 }  // namespace snd

@@ -308,7 +308,7 @@ cudaError_t chunk_post(const Plan& p, const ChunkPos& c, void* d_plane_out, cuda
 
 // kernels (launchers), each returns cudaGetLastError() of its launch and adds the number
 // of kernels it enqueued to p.launches
-cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cudaStream_t s);
+cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cudaStream_t s);  // also clears the block counters
 cudaError_t launch_tree(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream_t s);
 cudaError_t launch_mf(const Plan& p, int64_t e_prev, int64_t e_new, int64_t f_prev, int64_t f_new,
                       void* d_plane_out, cudaStream_t s);
@@ -346,8 +346,7 @@ cudaError_t launch_tree_direct_batch(const Plan* const* plans, const int64_t* e_
 template <typename Stage>
 cudaError_t chunk_post(const Plan& p, const ChunkPos& c, void* d_plane_out, cudaStream_t s, Stage&& stage) {
   cudaError_t e = cudaSuccess;
-  if (c.nb > 0) e = cudaMemsetAsync(p.dp.counters, 0, sizeof(uint32_t) * (kCntBlockCands + 1), s);
-  if (e == cudaSuccess && (c.nb > 0 || (d_plane_out && c.e_new > c.e_prev)))
+  if (c.nb > 0 || (d_plane_out && c.e_new > c.e_prev))
     e = stage(SND_STAGE_MF, [&] { return launch_mf(p, c.e_prev, c.e_new, c.f_prev, c.f_new, d_plane_out, s); });
   if (e == cudaSuccess && c.nb > 0)
     e = stage(SND_STAGE_CANDIDATES, [&] { return launch_candidates(p, c.f_prev, c.nb, s); });
