@@ -1,11 +1,10 @@
 // DM-scaled boxcar matched filter (Methods, "Matched filtering").
 //
 // One CTA per DM row. The row segment [F_prev, E_new) of the plane ring (block start times
-// [F_prev, F_new) plus the Wmax-1 samples their windows reach) is staged in shared memory,
-// realigned so that F_prev sits on a 16-byte boundary; its exact integer sums give mu and
-// sigma over the block's start times, and an in-place exclusive scan turns it into prefix
-// sums so every boxcar is P[t+W] - P[t]. Scan and threshold work on groups of four
-// consecutive samples per lane (one 128-bit shared access per group).
+// [F_prev, F_new) plus the Wmax-1 samples their windows reach) is staged in shared memory as it lies
+// in the ring (columns from the 16-byte boundary at or before F_prev); its exact integer sums give mu
+// and sigma over the block's start times, and an in-place exclusive scan turns it into prefix sums, so every boxcar is P[t+W] - P[t]. Everything works on quads of four consecutive
+// columns per lane (one 128-bit shared access).
 //
 // Decision: a cell is in the mask iff max over the row's widths of
 //   SNR(W) = (S_W - mu*W) / (sigma*sqrt(W))          (FP64, this operation order)
@@ -51,7 +50,6 @@ struct MfArgs {
   long long wait_cycles;  // bound of the staging wait (clock cycles)
 };
 
-constexpr int kMfThreads = 256;
 constexpr uint32_t kAllWidths = (1u << kNumWidthSlots) - 1u;
 
 template <bool A, bool NW = false>
@@ -64,171 +62,120 @@ __device__ __forceinline__ double snr_of(long long s, double mu_w, double den) {
   return __ddiv_rn(__dsub_rn(static_cast<double>(s), mu_w), den);
 }
 
-// One DM row d of one plan's block (the body of k_mf and of the many-beam k_mf_multi).
+// S/N in FP32 of a window sum: c = (bits of floor(mu W), its fraction, 1 / (sigma sqrt W))
+__device__ __forceinline__ float snr32(int s, const float3& c) {
+  return (static_cast<float>(s - __float_as_int(c.x)) - c.y) * c.z;
+}
+
+// One DM row d of one plan's block (the body of k_mf and of the many-beam k_mf_multi), by NT threads.
+//
+// What bounds it: shared-memory wavefronts (the threshold reads a quad per width and four start times)
+// and the latency of its phases one after the other, so the phases are few and touch shared memory
+// little: the copy lands, the quads are read once for the sums and once for the scan, which writes
+// them; the segment is never shifted to F_prev's column (the mask words are, at the end). Threads per
+// CTA follow the row's length, so that an SM's shared memory is full of threads.
+// Stage times before and after (us, with the event pair; before: a shifting pass, 256 threads, FP64 for
+// every width of a cell): 2048 rows x 16384 binary 113 -> 104, graded 132 -> 106, float with the caller's
+// plane 134 -> 113; 1537 x 10007 82 -> 63; 4096 x 7246 117 -> 95; 128 x 16384 59 -> 32.
+template <int NT>
 __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
-  // smem: 4 words of front pad, then y[0..4*G) with y 16-byte aligned, G = len/4 + 2 groups, and
-  // one spare group
-  extern __shared__ __align__(16) int32_t smem[];
-  constexpr int NWARP = kMfThreads / 32;
-  __shared__ long long red1[NWARP], red2[NWARP];
+  extern __shared__ __align__(16) int32_t smem[];  // G quads: columns ca0 .. of the ring, then prefix sums
+  constexpr int NW = NT / 32;
+  __shared__ long long red1[NW], red2[NW];
+  __shared__ uint32_t wsum[NW];
   __shared__ int tau[kNumWidthSlots];
   __shared__ double s_muw[kNumWidthSlots], s_den[kNumWidthSlots];
+  __shared__ float3 s_f32[kNumWidthSlots];
   __shared__ int s_ok;
-  __shared__ uint32_t wsum[NWARP];
+  __shared__ __align__(8) unsigned long long bar;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int len = static_cast<int>(a.e_new - a.f_prev);
   const int c0 = static_cast<int>(a.f_prev % a.Lp);
-  const int r0 = c0 & 3;
-  int32_t* y = smem + 4;  // y[i] = ring column c0 + i, zero from i = len on
-  int4* Y4 = reinterpret_cast<int4*>(y);
-  const int G = (len >> 2) + 2;  // groups staged: y[len] and one group past it
+  const int r0 = c0 & 3;               // staged column j holds sample j - r0 of the segment
+  const int G = ((len + r0) >> 2) + 1; // quads staged: up to the one whose first prefix may be P[len]
   const int nb = a.nb;
-  // groups of the statistics passes: warp 0 also finds the row's thresholds in FP64 (a long
-  // dependent chain), so the contiguous group segments go to warps 1..NWARP-1
-  constexpr int NSEG = NWARP - 1;
-  const int segg = ((G + NSEG * 32 - 1) / (NSEG * 32)) * 32;
-  const int glo = wid == 0 ? 0 : min(G, (wid - 1) * segg), ghi = wid == 0 ? 0 : min(G, glo + segg);
-  // 1. stage the row segment. Bulk path: the TMA engine copies ring columns c0 - r0 ... (16-byte
-  //    aligned) as they are, and the statistics pass below shifts them by sh = r0 in place, so
-  //    that y[i] = column c0 + i. Otherwise each thread loads and realigns its groups (sh = 0).
-  __shared__ int4 bnd[NWARP];  // first staged group of each warp's segment, before the shift
-  int sh = 0;
+  int4* Y4 = reinterpret_cast<int4*>(smem);
   const int32_t* src = a.plane + static_cast<size_t>(d) * a.Lp;
-  const int ng = G + (r0 != 0 ? 1 : 0);  // groups copied by the bulk path
-  if (4 * ng <= a.Lp) {
-    // one thread issues the bulk copies (one, or two across the ring's wrap point) onto an
-    // mbarrier; every thread waits for them (bounded)
-    __shared__ __align__(8) unsigned long long bar;
-    const uint32_t b = smem_u32(&bar);
-    if (tid == 0) {
-      bar_init(b, 1);
-      bar_init_fence();
-    }
-    __syncthreads();
-    const int ca0 = c0 - r0;
-    const int n1 = min(ng, (a.Lp - ca0) >> 2);  // groups before the wrap point
-    if (tid == 0) {
-      bar_expect(b, static_cast<uint32_t>(ng) * 16u);
-      bulk_g2s(smem_u32(y), src + ca0, static_cast<uint32_t>(n1) * 16u, b);
-      if (n1 < ng) bulk_g2s(smem_u32(y + 4 * n1), src, static_cast<uint32_t>(ng - n1) * 16u, b);
-    }
-    const bool ok = bar_wait(b, 0, a.wait_cycles);
-    if (!__syncthreads_and(ok)) {
-      // the wait gave up: report it, let the copies land (normal bound) before the CTA leaves
-      if (tid == 0) {
-        atomicOr(&a.counters[kCntStatus], kStatusMfTimeout);
-        bar_wait(b, 0, kStageWaitCycles);
-      }
-      return;
-    }
-    sh = r0;
-    if (lane == 0 && glo < ghi) bnd[wid] = Y4[glo];
-  } else {
-    // aligned group m of y takes global groups m and m+1 of the row (16-byte loads of columns
-    // c0 - r0 + 4m ...; Lp % 4 == 0, so a group never straddles the ring's wrap point); four
-    // groups per thread are loaded before any is stored, so their loads are in flight together
-    constexpr int KB = 4;
-    for (int m0 = tid; m0 < G; m0 += KB * kMfThreads) {
-      int4 g0[KB], g1[KB];
-#pragma unroll
-      for (int k = 0; k < KB; ++k) {
-        const int m = m0 + k * kMfThreads;
-        if (m >= G) break;
-        int ca = c0 - r0 + 4 * m;
-        if (ca >= a.Lp) ca -= a.Lp;
-        int cb = ca + 4;
-        if (cb >= a.Lp) cb -= a.Lp;
-        g0[k] = __ldg(reinterpret_cast<const int4*>(src + ca));
-        g1[k] = r0 != 0 ? __ldg(reinterpret_cast<const int4*>(src + cb)) : g0[k];
-      }
-#pragma unroll
-      for (int k = 0; k < KB; ++k) {
-        const int m = m0 + k * kMfThreads;
-        if (m >= G) break;
-        int4 o = g0[k];
-        if (r0 == 1) o = make_int4(g0[k].y, g0[k].z, g0[k].w, g1[k].x);
-        else if (r0 == 2) o = make_int4(g0[k].z, g0[k].w, g1[k].x, g1[k].y);
-        else if (r0 == 3) o = make_int4(g0[k].w, g1[k].x, g1[k].y, g1[k].z);
-        const int i = 4 * m;
-        if (i + 3 >= len) {
-          if (i >= len) o.x = 0;
-          if (i + 1 >= len) o.y = 0;
-          if (i + 2 >= len) o.z = 0;
-          if (i + 3 >= len) o.w = 0;
-        }
-        Y4[m] = o;
-      }
-    }
+  const int ca0 = c0 - r0;
+  // 1. one thread copies the segment (one bulk copy, or two across the ring's wrap point) onto an
+  //    mbarrier; every thread waits for it (bounded)
+  const uint32_t bs = smem_u32(&bar);
+  if (tid == 0) {
+    bar_init(bs, 1);
+    bar_init_fence();
   }
   __syncthreads();
-  // 2. one pass over each warp's segment: the shift by sh (bulk path) and the zero tail from
-  //    y[len] on, the caller's plane (the newly emitted samples [E_prev, E_new)), the segment's
-  //    total (for the scan) and the exact integer sums over the block's start times (y[i], i < nb)
-  const int first = static_cast<int>(a.e_prev - a.f_prev);
+  const int n1 = min(G, (a.Lp - ca0) >> 2);  // quads before the wrap point
+  if (tid == 0) {
+    bar_expect(bs, static_cast<uint32_t>(G) * 16u);
+    bulk_g2s(smem_u32(Y4), src + ca0, static_cast<uint32_t>(n1) * 16u, bs);
+    if (n1 < G) bulk_g2s(smem_u32(Y4 + n1), src, static_cast<uint32_t>(G - n1) * 16u, bs);
+  }
+  const bool landed = bar_wait(bs, 0, a.wait_cycles);
+  if (!__syncthreads_and(landed)) {
+    // the wait gave up: report it, let the copies land (normal bound) before the CTA leaves
+    if (tid == 0) {
+      atomicOr(&a.counters[kCntStatus], kStatusMfTimeout);
+      bar_wait(bs, 0, kStageWaitCycles);
+    }
+    return;
+  }
+  // 2. one pass over the warp's quads (contiguous per warp), which are zero outside the segment: the
+  //    caller's plane (the newly emitted samples [E_prev, E_new)), the exact sums over the block's start
+  //    times and the warp's total for the scan
+  const int seg = (((G + 31) >> 5) + NW - 1) / NW * 32;
+  const int glo = min(G, wid * seg), ghi = min(G, glo + seg);
+  auto quad = [&](int g) {
+    int4 v = Y4[g];
+    const int i = 4 * g - r0;  // sample of the quad's first column
+    if (i < 0 || i + 3 >= len) {
+      if (i < 0 || i >= len) v.x = 0;
+      if (i + 1 < 0 || i + 1 >= len) v.y = 0;
+      if (i + 2 < 0 || i + 2 >= len) v.z = 0;
+      if (i + 3 >= len) v.w = 0;
+    }
+    return v;
+  };
+  if (a.plane_out) {
+    // lanes along the row, one column each, so a store instruction covers 32 neighbouring values
+    const int j0 = static_cast<int>(a.e_prev - a.f_prev) + r0;  // staged column of the first emitted sample
+    const int32_t* y = smem + j0;
+    const size_t o = static_cast<size_t>(d) * a.nemit;
+    if (a.out_scale != 0.0f) {
+      float* out = static_cast<float*>(a.plane_out) + o;
+      for (int k = tid; k < a.nemit; k += NT) out[k] = static_cast<float>(y[k]) * a.out_scale;
+    } else if (a.out_u8) {
+      uint8_t* out = static_cast<uint8_t*>(a.plane_out) + o;
+      for (int k = tid; k < a.nemit; k += NT) out[k] = static_cast<uint8_t>(y[k]);
+    } else {
+      int32_t* out = static_cast<int32_t*>(a.plane_out) + o;
+      for (int k = tid; k < a.nemit; k += NT) out[k] = y[k];
+    }
+  }
+  if (nb <= 0) return;
   {
     uint32_t tot = 0;
     long long s1 = 0, s2 = 0;
-    // a lane sums y and y^2 in 32 bits where its groups cannot overflow them (a.stat32), else
-    // in 64 bits; the warp reduction is in 64 bits either way
+    // a lane sums y and y^2 in 32 bits where its quads cannot overflow them (a.stat32), else in
+    // 64 bits; the warp reduction is in 64 bits either way
     auto pass = [&](auto zero) {
       using Acc = decltype(zero);
       Acc a1 = 0, a2 = 0;
-      for (int base = glo; base < ghi; base += 32) {
-        const int g = base + lane;
-        int4 v = make_int4(0, 0, 0, 0);
-        if (g < ghi) {
-          v = Y4[g];
-          if (sh != 0) {
-            // y group g = the last 4 - sh values of staged group g and the first sh of group g + 1
-            // (the next warp's first group as it was before that warp shifted it)
-            const int4 nx = (g + 1 == ghi && g + 1 < G) ? bnd[wid + 1] : Y4[g + 1];
-            if (sh == 1) v = make_int4(v.y, v.z, v.w, nx.x);
-            else if (sh == 2) v = make_int4(v.z, v.w, nx.x, nx.y);
-            else v = make_int4(v.w, nx.x, nx.y, nx.z);
-          }
-          const int i = 4 * g;
-          if (i + 3 >= len) {
-            if (i >= len) v.x = 0;
-            if (i + 1 >= len) v.y = 0;
-            if (i + 2 >= len) v.z = 0;
-            if (i + 3 >= len) v.w = 0;
-          }
-        }
-        if (sh != 0) __syncwarp();  // every lane has read its next group before any is rewritten
-        if (g < ghi && (sh != 0 || 4 * g + 3 >= len)) Y4[g] = v;
-        if (g >= ghi) continue;
-        const int i = 4 * g;
-        if (a.plane_out && i + 3 >= first && i < first + a.nemit) {
-          const int vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int k = i + e - first;
-            if (k < 0 || k >= a.nemit) continue;
-            const size_t o = static_cast<size_t>(d) * a.nemit + k;
-            if (a.out_scale != 0.0f) static_cast<float*>(a.plane_out)[o] = static_cast<float>(vv[e]) * a.out_scale;
-            else if (a.out_u8) static_cast<uint8_t*>(a.plane_out)[o] = static_cast<uint8_t>(vv[e]);
-            else static_cast<int32_t*>(a.plane_out)[o] = vv[e];
-          }
-        }
+#pragma unroll 2
+      for (int g = glo + lane; g < ghi; g += 32) {
+        const int4 v = quad(g);
+        const int i = 4 * g - r0;
+        const Acc x = static_cast<Acc>(v.x), y = static_cast<Acc>(v.y), z = static_cast<Acc>(v.z), w = static_cast<Acc>(v.w);
         const uint32_t gs = static_cast<uint32_t>(v.x) + static_cast<uint32_t>(v.y) + static_cast<uint32_t>(v.z) +
                             static_cast<uint32_t>(v.w);
         tot += gs;
-        const Acc vx = static_cast<Acc>(v.x), vy = static_cast<Acc>(v.y), vz = static_cast<Acc>(v.z),
-                  vw = static_cast<Acc>(v.w);
-        if (i + 3 < nb) {
+        if (i + 3 < nb) {  // columns before the segment are zero
           a1 += static_cast<Acc>(gs);
-          a2 += (vx * vx + vy * vy) + (vz * vz + vw * vw);
-        } else if (i < nb) {
-          a1 += vx;
-          a2 += vx * vx;
-          if (i + 1 < nb) {
-            a1 += vy;
-            a2 += vy * vy;
-          }
-          if (i + 2 < nb) {
-            a1 += vz;
-            a2 += vz * vz;
-          }
+          a2 += (x * x + y * y) + (z * z + w * w);
+        } else {
+          if (i < nb) { a1 += x; a2 += x * x; }
+          if (i + 1 < nb) { a1 += y; a2 += y * y; }
+          if (i + 2 < nb) { a1 += z; a2 += z * z; }
         }
       }
       s1 = static_cast<long long>(a1);
@@ -248,12 +195,11 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
     }
   }
   __syncthreads();
-  if (nb <= 0) return;
   const uint32_t wm = a.width_mask[d];
-  if (wid == 0) {
+  if (wid == NW - 1) {
     // row statistics (FP64, fixed order) and, lane j, the integer threshold of width 2^j
     long long t1 = 0, t2 = 0;
-    for (int w = 0; w < NWARP; ++w) {
+    for (int w = 0; w < NW; ++w) {
       t1 += red1[w];
       t2 += red2[w];
     }
@@ -269,6 +215,9 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
       const double den = __dmul_rn(sig, __dsqrt_rn(w));
       s_muw[lane] = mu_w;
       s_den[lane] = den;
+      const double whole = floor(mu_w);
+      s_f32[lane] = make_float3(__int_as_float(static_cast<int>(whole)), static_cast<float>(mu_w - whole),
+                                static_cast<float>(1.0 / den));
       double est = ceil(__dadd_rn(mu_w, __dmul_rn(a.theta, den)));
       if (est < 0.0) est = 0.0;
       if (est > 2147483000.0) est = 2147483000.0;
@@ -286,15 +235,14 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
       tau[lane] = static_cast<int>(sv);
     }
   }
-  // 3. exclusive scan in place (uint32 wrap-around keeps window sums exact): a lane scans its
-  //    group of four, the warp scans the group totals, the running carry starts at the sum of
-  //    the segments before this warp's
+  // 3. exclusive scan in place (uint32 wrap-around keeps window sums exact): a lane scans its quad, the
+  //    warp scans the quads' sums, the running carry starts at the sum of the warps before
   {
     uint32_t carry = 0;
     for (int w = 0; w < wid; ++w) carry += wsum[w];
     for (int base = glo; base < ghi; base += 32) {
       const int g = base + lane;
-      const int4 v = (g < ghi) ? Y4[g] : make_int4(0, 0, 0, 0);
+      const int4 v = g < ghi ? quad(g) : make_int4(0, 0, 0, 0);
       const uint32_t a0 = static_cast<uint32_t>(v.x);
       const uint32_t a1 = a0 + static_cast<uint32_t>(v.y);
       const uint32_t a2 = a1 + static_cast<uint32_t>(v.z);
@@ -317,36 +265,32 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
   // across the wrap point) while this row is scored
   if (tid == 0 && d + a.pf_rows < a.ndm) {
     const int32_t* nsrc = a.plane + static_cast<size_t>(d + a.pf_rows) * a.Lp;
-    const int gq = min(G + 1, a.Lp >> 2);  // 16-byte groups of the next row's staged columns
-    const int n1 = min(gq, (a.Lp - (c0 - r0)) >> 2);
-    bulk_prefetch_l2(nsrc + (c0 - r0), static_cast<uint32_t>(n1) * 16u);
-    if (n1 < gq) bulk_prefetch_l2(nsrc, static_cast<uint32_t>(gq - n1) * 16u);
+    bulk_prefetch_l2(nsrc + ca0, static_cast<uint32_t>(n1) * 16u);
+    if (n1 < G) bulk_prefetch_l2(nsrc, static_cast<uint32_t>(G - n1) * 16u);
   }
   const int nbw = (nb + 31) >> 5;
   uint32_t* mrow = a.mask + static_cast<size_t>(d) * a.mw;
   if (!s_ok) {
-    for (int q = tid; q < nbw; q += kMfThreads) mrow[q] = 0;
+    for (int q = tid; q < nbw; q += NT) mrow[q] = 0;
     return;
   }
   int tw[kNumWidthSlots];
 #pragma unroll
   for (int j = 0; j < kNumWidthSlots; ++j) tw[j] = ((wm >> j) & 1) ? tau[j] : 0x7FFFFFFF;
-  const uint32_t* P = reinterpret_cast<const uint32_t*>(y);
-  const uint4* P4 = reinterpret_cast<const uint4*>(y);
-  // 4. threshold: lane m of an iteration tests start times 4m..4m+3 against every width of the
-  //    row (window ends P[4m + W ...] are group m + W/4 for W >= 4, groups m and m+1 below).
+  const uint32_t* P = reinterpret_cast<const uint32_t*>(smem) + r0;  // P[t]: the sum before sample t
+  const uint4* P4 = reinterpret_cast<const uint4*>(smem);
+  // 4. threshold: lane m of an iteration tests the start times of quad m against every width of the
+  //    row (window ends P[4m + W ...] are quad m + W/4 for W >= 4, quads m and m+1 below).
   //    A cell passes iff max over widths of S_W - tau_W >= 0; S_W < 2^31 and tau_W < 2^31, so
-  //    the wrapped difference P[t+W] - P[t] - tau_W read as int32 is exact. Eight lanes'
-  //    nibbles make one mask word.
-  // hit nibble of start times 4m..4m+3 (bit e: start time 4m + e passes)
+  //    the wrapped difference P[t+W] - P[t] - tau_W read as int32 is exact.
+  // hit nibble of quad m (bit e: its column e passes)
   // Without wrap-around (prefix sums below 2^31, the usual case) the test is rearranged as
   // max over W of (P[t+W] - tau_W) >= P[t]: one add-and-max per (start time, width), which
   // the compiler can issue as a single three-input integer instruction.
-  auto group_hits = [&](int m, auto all) -> uint32_t {
+  auto quad_hits = [&](int m, auto all) -> uint32_t {
     constexpr bool ALL = decltype(all)::kAll;
     constexpr bool NOWRAP = decltype(all)::kNoWrap;
-    const uint4 p = P4[m];
-    const uint4 q = P4[m + 1];
+    const uint4 p = P4[m], q = P4[m + 1];
     int h0 = INT_MIN, h1 = INT_MIN, h2 = INT_MIN, h3 = INT_MIN;
     auto upd = [](int& h, uint32_t end, uint32_t start, int tj) {
       if constexpr (NOWRAP) {
@@ -373,54 +317,67 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
       upd(h2, q.z, p.z, tw[2]);
       upd(h3, q.w, p.w, tw[2]);
     }
-    auto wide = [&](int j) {
-      const uint4 e = P4[m + (1 << (j - 2))];
-      upd(h0, e.x, p.x, tw[j]);
-      upd(h1, e.y, p.y, tw[j]);
-      upd(h2, e.z, p.z, tw[j]);
-      upd(h3, e.w, p.w, tw[j]);
-    };
 #pragma unroll
     for (int j = 3; j < kNumWidthSlots; ++j)
-      if (ALL || ((wm >> j) & 1u)) wide(j);
+      if (ALL || ((wm >> j) & 1u)) {
+        const uint4 e = P4[m + (1 << (j - 2))];
+        upd(h0, e.x, p.x, tw[j]);
+        upd(h1, e.y, p.y, tw[j]);
+        upd(h2, e.z, p.z, tw[j]);
+        upd(h3, e.w, p.w, tw[j]);
+      }
     if constexpr (NOWRAP)
       return (h0 >= static_cast<int>(p.x) ? 1u : 0u) | (h1 >= static_cast<int>(p.y) ? 2u : 0u) |
              (h2 >= static_cast<int>(p.z) ? 4u : 0u) | (h3 >= static_cast<int>(p.w) ? 8u : 0u);
     return (h0 >= 0 ? 1u : 0u) | (h1 >= 0 ? 2u : 0u) | (h2 >= 0 ? 4u : 0u) | (h3 >= 0 ? 8u : 0u);
   };
-  const int ngt = (nb + 3) >> 2;
-  for (int base = wid * 32; base < ngt; base += NWARP * 32) {
-    const int m = base + lane;
+  // The warps take iterations in turn (a burst's cells, which cost an evaluation each, spread over
+  // them). An iteration makes four column words (word k = columns 32 k ..), kept in the mask row until
+  // all are there; the mask word of start times 32 q .. is column words q and q + 1 shifted by r0.
+  const int tit = (nb + r0 + 127) >> 7;  // iterations over the columns of start times
+  for (int it = wid; it < tit; it += NW) {
+    const int m = it * 32 + lane;
+    const int i = 4 * m - r0;  // start time of the quad's first column
     uint32_t nib = 0;
-    if (m < ngt) {
+    if (i + 3 >= 0 && i < nb) {
       // rows with every width (most rows above a small DM) take a copy of the loop with no
-      // width tests, so all window loads of the group can be in flight together
+      // width tests, so all window loads of the quad can be in flight together
       if (a.nowrap)
-        nib = (wm == kAllWidths) ? group_hits(m, WidthSet<true, true>{}) : group_hits(m, WidthSet<false, true>{});
+        nib = (wm == kAllWidths) ? quad_hits(m, WidthSet<true, true>{}) : quad_hits(m, WidthSet<false, true>{});
       else
-        nib = (wm == kAllWidths) ? group_hits(m, WidthSet<true>{}) : group_hits(m, WidthSet<false>{});
-      const int rem = nb - 4 * m;  // start times of this group inside the block
-      if (rem < 4) nib &= (1u << rem) - 1u;
+        nib = (wm == kAllWidths) ? quad_hits(m, WidthSet<true>{}) : quad_hits(m, WidthSet<false>{});
+      if (nb - i < 4) nib &= (1u << (nb - i)) - 1u;  // start times inside the block
+      if (i < 0) nib &= ~((1u << -i) - 1u);
     }
     uint32_t word = nib << (4 * (lane & 7));
     word |= __shfl_xor_sync(0xFFFFFFFFu, word, 1);
     word |= __shfl_xor_sync(0xFFFFFFFFu, word, 2);
     word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
-    const int qw = (base >> 3) + (lane >> 3);
-    if ((lane & 7) == 0 && qw < nbw) mrow[qw] = word;
+    const int k = 4 * it + (lane >> 3);
+    if ((lane & 7) == 0 && k <= nbw) mrow[k] = word;  // a mask row has a word past its last (96 spare columns)
     while (nib) {
       const int e = __ffs(nib) - 1;
       nib &= nib - 1u;
-      const int t = 4 * m + e;
+      const int t = i + e;
       const uint32_t p0 = P[t];
+      // The cell's S/N is the FP64 maximum over the widths. FP64 divides are slow here, so FP32 finds
+      // the widths that can hold it: S - floor(mu W) is an exact integer, and what is left rounds to
+      // a few 1e-7 of a value above Theta, so a width more than 1e-4 below the largest cannot.
+      float best32 = -3.0e38f;
+#pragma unroll
+      for (int j = 0; j < kNumWidthSlots; ++j)
+        if ((wm >> j) & 1) best32 = fmaxf(best32, snr32(static_cast<int>(P[t + (1 << j)] - p0), s_f32[j]));
+      const float floor32 = best32 - 1e-4f * fabsf(best32);
       double best = -1.0e300;
       int bw = 0;
+#pragma unroll 1
       for (int j = 0; j < kNumWidthSlots; ++j) {
         if (!((wm >> j) & 1)) continue;
-        const long long S = static_cast<int>(P[t + (1 << j)] - p0);
-        const double v = snr_of(S, s_muw[j], s_den[j]);
-        if (v > best) {
-          best = v;
+        const int S = static_cast<int>(P[t + (1 << j)] - p0);
+        if (!(snr32(S, s_f32[j]) >= floor32)) continue;
+        const double sv = snr_of(S, s_muw[j], s_den[j]);
+        if (sv > best) {
+          best = sv;
           bw = 1 << j;
         }
       }
@@ -436,9 +393,18 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
       }
     }
   }
+  if (r0 == 0) return;
+  __syncthreads();
+  for (int q0 = 0; q0 < nbw; q0 += NT) {
+    const int q = q0 + tid;
+    const uint32_t w = q < nbw ? __funnelshift_r(mrow[q], q + 1 < 4 * tit ? mrow[q + 1] : 0u, r0) : 0u;
+    __syncthreads();  // every word of this round is read before one is rewritten
+    if (q < nbw) mrow[q] = w;
+  }
 }
 
-__global__ void __launch_bounds__(kMfThreads, 3) k_mf(const __grid_constant__ MfArgs a) { mf_row(a, blockIdx.x); }
+template <int NT>
+__global__ void __launch_bounds__(NT, 1152 / NT) k_mf(const __grid_constant__ MfArgs a) { mf_row<NT>(a, blockIdx.x); }
 
 constexpr int kMaxMfBeams = 64;
 
@@ -450,20 +416,41 @@ struct MfMulti {
   MfArgs beam[kMaxMfBeams];
 };
 
-__global__ void __launch_bounds__(kMfThreads, 3) k_mf_multi(const __grid_constant__ MfMulti m) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 1152 / NT) k_mf_multi(const __grid_constant__ MfMulti m) {
   const int i = static_cast<int>(blockIdx.x);
   int lo = 0, hi = m.nbeams - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (m.first[mid] <= i) lo = mid; else hi = mid - 1;
   }
-  mf_row(m.beam[lo], i - m.first[lo]);
+  mf_row<NT>(m.beam[lo], i - m.first[lo]);
 }
 
-// Arguments of one plan's block; *smem = the dynamic shared memory of its row staging.
+// Threads per CTA by how many CTAs' rows fit an SM (four and more: 256; three: 384; two: 512; one:
+// 1024), or 1024 where the rows are too few to fill the GPU (`alone`: at most one per SM).
+enum { kMf256, kMf384, kMf512, kMf1024, kMfShapes };
+int mf_shape(int quads, bool alone) {
+  const int smem = quads * 16 + 2048;
+  if (alone && quads > 1024) return kMf1024;
+  if (smem <= 56 * 1024) return kMf256;
+  if (smem <= 75 * 1024) return kMf384;
+  return smem <= 113 * 1024 ? kMf512 : kMf1024;
+}
+template <typename F>
+cudaError_t mf_dispatch(int shape, F&& f) {
+  switch (shape) {
+    case kMf256: return f.template go<256>();
+    case kMf384: return f.template go<384>();
+    case kMf512: return f.template go<512>();
+    default: return f.template go<1024>();
+  }
+}
+
+// Arguments of one plan's block; *quads = the quads of a row's segment.
 // Returns false when the block has nothing to do.
 bool mf_args(const Plan& p, int64_t e_prev, int64_t e_new, int64_t f_prev, int64_t f_new, void* d_plane_out,
-             MfArgs& a, int* smem) {
+             MfArgs& a, int* quads) {
   const int nb = static_cast<int>(f_new - f_prev);
   const int nemit = static_cast<int>(e_new - e_prev);
   if (nb <= 0 && (d_plane_out == nullptr || nemit <= 0)) return false;
@@ -490,81 +477,87 @@ bool mf_args(const Plan& p, int64_t e_prev, int64_t e_new, int64_t f_prev, int64
   a.out_u8 = p.plane_u8;
   a.tau_steps = p.loop_limit > 0 ? static_cast<int>(p.loop_limit < 64 ? p.loop_limit : 64) : 64;
   const int len = static_cast<int>(e_new - f_prev);
-  *smem = ((len >> 2) + 4) * 16;  // front pad (4 words), len/4 + 2 aligned groups and one more for the
-                                  // bulk copy of a segment that starts off a 16-byte boundary
+  *quads = ((len + static_cast<int>(f_prev % p.Lp & 3)) >> 2) + 1;  // as mf_row stages them
   {
     // largest root value of the mode times the staged samples bounds every prefix sum
     const double vmax = p.mode == SND_MODE_BINARY ? 1.0 : (p.mode == SND_MODE_GRADED ? p.N : p.nchan);
     a.nowrap = vmax * (len + 8.0) < 2147483647.0 ? 1 : 0;
-    // samples a lane of the statistics pass sums (its groups of the seven-warp segments)
-    const int groups = (len >> 2) + 2;
-    const double per_lane = 4.0 * ((groups + 7 * 32 - 1) / (7 * 32));
+    // samples a lane of the statistics sums (at least 256 threads)
+    const double per_lane = 4.0 * ((*quads + 255) / 256);
     a.stat32 = per_lane * vmax * vmax < 4294967295.0 ? 1 : 0;
   }
   a.wait_cycles = p.wait_limit > 0 ? p.wait_limit : kStageWaitCycles;
   return true;
 }
 
-// rows resident at once on the GPU for a kernel with `smem` bytes per CTA
-template <typename K>
-cudaError_t resident_rows(K kern, int smem, int fallback, int* out) {
-  int dev = 0, nsm = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMfThreads, smem);
-  *out = per_sm > 0 ? nsm * per_sm : fallback;
-  return e;
-}
+// The launch of one shape: the rows of one plan or of many.
+struct MfLaunch {
+  MfArgs* one;
+  MfMulti* many;
+  int rows, smem;
+  cudaStream_t s;
+  template <int NT>
+  cudaError_t go() {
+    const void* kern = many ? reinterpret_cast<const void*>(k_mf_multi<NT>) : reinterpret_cast<const void*>(k_mf<NT>);
+    int dev = 0, nsm = 0, per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+    if (e != cudaSuccess) return e;
+    const int resident = per_sm > 0 ? nsm * per_sm : rows;  // rows in flight: the next wave's are prefetched
+    if (many) {
+      for (int b = 0; b < many->nbeams; ++b) many->beam[b].pf_rows = resident;
+      k_mf_multi<NT><<<rows, NT, smem, s>>>(*many);
+    } else {
+      one->pf_rows = resident;
+      k_mf<NT><<<rows, NT, smem, s>>>(*one);
+    }
+    return cudaGetLastError();
+  }
+};
 
 }  // namespace
 
 cudaError_t launch_mf(const Plan& p, int64_t e_prev, int64_t e_new, int64_t f_prev, int64_t f_new,
                       void* d_plane_out, cudaStream_t s) {
   MfArgs a;
-  int smem = 0;
-  if (!mf_args(p, e_prev, e_new, f_prev, f_new, d_plane_out, a, &smem)) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_mf, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) e = resident_rows(k_mf, smem, p.ndm, &a.pf_rows);
+  int quads = 0;
+  if (!mf_args(p, e_prev, e_new, f_prev, f_new, d_plane_out, a, &quads)) return cudaSuccess;
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  k_mf<<<p.ndm, kMfThreads, smem, s>>>(a);
   p.launches += 1;
-  return cudaGetLastError();
+  return mf_dispatch(mf_shape(quads, p.ndm <= nsm), MfLaunch{&a, nullptr, p.ndm, quads * 16, s});
 }
 
 cudaError_t launch_mf_batch(const Plan* const* plans, const ChunkPos* pos, int n, cudaStream_t s) {
-  // Blocks are grouped by the CTAs per SM their row staging allows (shared memory up to about
-  // 72 KB: three, 110 KB: two, more: one), so a long-chunk beam does not lower the occupancy of
-  // every other beam's rows: at most three launches (more only past 64 beams per group).
-  auto cls = [](int smem) { return smem <= 72 * 1024 ? 0 : (smem <= 110 * 1024 ? 1 : 2); };
+  // Blocks are grouped by their rows' shape, so a long-chunk beam does not lower the occupancy of
+  // every other beam's rows: a launch per shape in use (more only past 64 beams of one).
   std::vector<MfArgs> args(n);
-  std::vector<int> sm(n, 0), live(n, 0);
+  std::vector<int> quads(n, 0), live(n, 0);
   for (int i = 0; i < n; ++i)
-    live[i] = mf_args(*plans[i], pos[i].e_prev, pos[i].e_new, pos[i].f_prev, pos[i].f_new, nullptr, args[i], &sm[i]);
-  for (int c = 0; c < 3; ++c) {
+    live[i] = mf_args(*plans[i], pos[i].e_prev, pos[i].e_new, pos[i].f_prev, pos[i].f_new, nullptr, args[i], &quads[i]);
+  for (int c = 0; c < kMfShapes; ++c) {
     for (int i0 = 0; i0 < n;) {
       MfMulti m{};
-      int smem = 0, ctas = 0;
+      int most = 0, rows = 0;
       const Plan* owner = nullptr;
       int i = i0;
       for (; i < n && m.nbeams < kMaxMfBeams; ++i) {
-        if (!live[i] || cls(sm[i]) != c) continue;
+        if (!live[i] || mf_shape(quads[i], false) != c) continue;
         m.beam[m.nbeams] = args[i];
-        m.first[m.nbeams] = ctas;
-        ctas += plans[i]->ndm;
-        smem = smem > sm[i] ? smem : sm[i];
+        m.first[m.nbeams] = rows;
+        rows += plans[i]->ndm;
+        most = most > quads[i] ? most : quads[i];
         if (!owner) owner = plans[i];
         ++m.nbeams;
       }
       i0 = i;
       if (m.nbeams == 0) continue;
-      cudaError_t e = cudaFuncSetAttribute(k_mf_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      int pf = 0;
-      if (e == cudaSuccess) e = resident_rows(k_mf_multi, smem, ctas, &pf);
-      if (e != cudaSuccess) return e;
-      for (int b = 0; b < m.nbeams; ++b) m.beam[b].pf_rows = pf;
-      k_mf_multi<<<ctas, kMfThreads, smem, s>>>(m);
       owner->launches += 1;
-      e = cudaGetLastError();
+      const cudaError_t e = mf_dispatch(c, MfLaunch{nullptr, &m, rows, most * 16, s});
       if (e != cudaSuccess) return e;
     }
   }
