@@ -1,5 +1,5 @@
 // Shared-memory staging primitives of the sm_103a kernels: mbarriers with bounded waits and
-// bulk (TMA engine) copies from global memory, in inline PTX.
+// bulk (TMA engine) copies from global memory, and shared-memory loads by address, in inline PTX.
 #pragma once
 
 #include <stdint.h>
@@ -63,6 +63,15 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
+}
+
+// 32-bit load at a shared-memory byte address plus a constant: one instruction, where a generic pointer
+// costs its address arithmetic again for every unrolled use
+template <int OFF>
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1 + %2];" : "=r"(v) : "r"(addr), "n"(OFF));
+  return v;
 }
 
 // bulk prefetch of global memory into L2 (16-byte aligned address, size a multiple of 16)

@@ -331,7 +331,7 @@ int build_plan(Plan& p) {
   p.off.gmeta = take(sizeof(uint32_t) * p.gmeta.size());
   p.off.tile_wb = take(sizeof(int32_t) * p.tile_wb.size());
   p.off.delays = take(sizeof(int32_t) * p.delays.size());
-  p.off.dmeta = take(sizeof(uint16_t) * std::max<size_t>(8, p.dmeta.size()));
+  p.off.dmeta = take(sizeof(uint32_t) * std::max<size_t>(4, p.dmeta.size()));
   p.off.dbase = take(sizeof(int32_t) * std::max<size_t>(4, p.dbase.size()));
   p.off.level_fires = take(sizeof(unsigned long long) * snd::kMaxLevels);
   if (p.mode == SND_MODE_ZFLOAT) {
@@ -520,8 +520,9 @@ int choose_tree_geometry_w(Plan& p, int warps) {
 // tile shape, and its tables. A CTA covers 32 consecutive trial DMs (lanes) and warps x kw
 // output words; channels are staged 64 at a time. Per (DM tile, channel) the first staged ring
 // word is base4 = (min over the tile of delta >> 5) rounded down to a multiple of 4 (16-byte
-// aligned bulk copies), and per (tile, channel, DM) the 16-bit entry (delta >> 5) - base4 << 5 |
-// delta & 31 gives the DM's window word and funnel shift.
+// aligned bulk copies), and per (tile, channel, DM) the entry (byte offset of window word
+// (delta >> 5) - base4 among the windows of the channel's round) << 5 | delta & 31 gives the DM's
+// window word and funnel shift.
 void choose_direct_geometry(Plan& p) {
   snd::DirectGeom& g = p.dgeom;
   g = snd::DirectGeom{};
@@ -631,25 +632,26 @@ void choose_direct_geometry(Plan& p) {
   if (omax > 2047) return;
   g.cspan = static_cast<int>(align_up(static_cast<size_t>(4 + omax + g.warps * span_kw), 4));
   // stage 128 channels per round (half the barriers) when they fit two CTAs per SM
-  auto smem_for = [&](int sg) { return (2 * 64 * sg * static_cast<int64_t>(g.cspan) + 64 * sg * 32 + nc) * 4; };
+  auto smem_for = [&](int sg) { return (2 * 64 * sg * (static_cast<int64_t>(g.cspan) + 32) + nc) * 4; };
   if (p.tree_round == 64)
     g.sgroups = 1;
   else if (p.tree_round == 128)
     g.sgroups = nc % 128 == 0 ? 2 : 1;
   else
-    g.sgroups = (nc % 128 == 0 && smem_for(2) <= 100 * 1024) ? 2 : 1;
+    g.sgroups = (nc % 128 == 0 && smem_for(2) <= 112 * 1024) ? 2 : 1;
   const int64_t smem = smem_for(g.sgroups);
-  if (smem > 200 * 1024) return;
+  if (smem > 220 * 1024) return;
   g.smem_bytes = static_cast<int>(smem);
   p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nc * 32, 0);
   for (int t = 0; t < g.ndm_tiles; ++t)
-    for (int c = 0; c < nchan; ++c) {
+    for (int c = 0; c < nc; ++c) {
       const int32_t b4 = p.dbase[static_cast<size_t>(t) * nc + c];
       for (int l = 0; l < 32; ++l) {
         const int d = std::min(ndm - 1, t * 32 + l);
-        const int32_t v = p.delays[static_cast<size_t>(d) * nchan + c];
-        p.dmeta[(static_cast<size_t>(t) * nc + c) * 32 + l] =
-            static_cast<uint16_t>((((v >> 5) - b4) << 5) | (v & 31));
+        // channels past the last read their own (zero) row at any delay
+        const int32_t v = c < nchan ? p.delays[static_cast<size_t>(d) * nchan + c] : 0;
+        const uint32_t at = static_cast<uint32_t>((c % (64 * g.sgroups)) * g.cspan + (v >> 5) - b4);
+        p.dmeta[(static_cast<size_t>(t) * nc + c) * 32 + l] = (at * 4) << 5 | static_cast<uint32_t>(v & 31);
       }
     }
   g.inst = inst;

@@ -170,7 +170,7 @@ struct DevPtrs {
   int32_t* zeoff;          // zfloat: [ndm_tiles][nleaves + 1] first pattern of each (tile, leaf)
   int32_t* zent;           // zfloat: [patterns][8] window offset of each channel | (its first delay mod 8) << 28; [7]: leaf << 16 | span
   uint32_t* zdm;           // zfloat: [ndm_tiles][nleaves][16] pattern in the tile << 14 | delay past the pattern's first
-  uint16_t* dmeta;         // direct tree: [ndm_tiles][nchan][32] staged word offset << 5 | shift
+  uint32_t* dmeta;         // direct tree: [ndm_tiles][nchan][32] byte offset in a round's windows << 5 | shift
   int32_t* dbase;          // direct tree: [ndm_tiles][nchan] first staged ring word (multiple of 4)
   unsigned long long* level_fires;  // [kMaxLevels] firing node-samples per tree level (SND_FLAG_LEVEL_RATES)
 };
@@ -235,7 +235,7 @@ struct Plan {
   TreeGeom geom{};
   DirectGeom dgeom{};
   bool direct = false;                  // the tree runs on the direct kernel (tree_direct.cu)
-  std::vector<uint16_t> dmeta;
+  std::vector<uint32_t> dmeta;
   std::vector<int32_t> dbase;
   ZGeom zgeom{};
   std::vector<int32_t> zwb, zcarry, zeoff, zent;

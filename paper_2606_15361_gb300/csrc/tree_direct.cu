@@ -19,8 +19,10 @@
 //
 // GPU mapping:
 //  * lanes are 32 consecutive trial DMs; a warp owns KW consecutive 32-sample words of the
-//    CTA's time tile (warp w: words w*KW ..), so per channel a lane reads one 16-bit offset
-//    and then KW+1 consecutive window words (a sliding funnel-shift window). The 32 DMs of a
+//    CTA's time tile (warp w: words w*KW ..), so per channel a lane reads one table entry (its byte
+//    offset among the round's windows and the bit shift: one add gives the address; a 16-bit word
+//    offset per channel took three instructions) and then KW+1 consecutive window words (a sliding
+//    funnel-shift window). The 32 DMs of a
 //    tile read one channel at offsets that differ by less than 32 words, so the reads hit
 //    distinct banks (or broadcast) without conflicts.
 //  * channels are staged 64 or 128 at a time (a round): every warp issues TMA bulk copies
@@ -49,7 +51,7 @@ struct DirArgs {
   int level_nodes[kMaxLevels];
   int sub_groups;          // graded: staged groups per exact-level node
   int sub_lev;             // graded: the exact level
-  const uint16_t* meta;    // [ndm_tiles][nchan][32]: (word offset << 5) | bit shift
+  const uint32_t* meta;    // [ndm_tiles][nchan][32]: (byte offset in the round's windows << 5) | bit shift
   const int32_t* base4;    // [ndm_tiles][nchan]: first staged ring word (relative, multiple of 4)
   int cspan;               // staged words per channel (multiple of 4)
   int sgroups;             // adder groups of kDG channels staged per round (1 or 2)
@@ -581,8 +583,8 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
   const int SG = kDG * a.sgroups;                  // channels per staging round
   const int wbuf = SG * cspan;                     // window words per buffer
   uint32_t* win = sm;                              // [2][SG][cspan]
-  uint16_t* met = reinterpret_cast<uint16_t*>(sm + 2 * wbuf);  // [2][SG][32]
-  int32_t* sbase = reinterpret_cast<int32_t*>(sm + 2 * wbuf + SG * 32);  // [nchan]
+  uint32_t* met = sm + 2 * wbuf;                   // [2][SG][32]
+  int32_t* sbase = reinterpret_cast<int32_t*>(sm + 2 * wbuf + 2 * SG * 32);  // [nchan]
   const long long aw0 = a.word0 + static_cast<long long>(bx) * a.tile_words;
   const int lead = static_cast<int>(aw0 & 3);
   const long long aw4 = aw0 - lead;
@@ -612,7 +614,7 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     // the buffer's previous contents were read by every warp before the last barrier
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (lane == 0)
-      bar_expect(bar, static_cast<uint32_t>((i1 > i0 ? i1 - i0 : 0) * cspan * 4 + (wd == 0 ? SG * 64 : 0)));
+      bar_expect(bar, static_cast<uint32_t>((i1 > i0 ? i1 - i0 : 0) * cspan * 4 + (wd == 0 ? SG * 128 : 0)));
     __syncwarp();
     for (int i = i0 + lane; i < i1; i += 32) {
       const int c = g * SG + i;
@@ -621,7 +623,7 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     }
     if (wd == 0 && lane == 0)
       bulk_g2s(smem_u32(met + b * SG * 32), a.meta + (static_cast<size_t>(tile) * a.nchan + g * SG) * 32,
-               static_cast<uint32_t>(SG * 64), bar);
+               static_cast<uint32_t>(SG * 128), bar);
   };
 
   DState<MODE, KW, NPL, MAXU> st;
@@ -639,14 +641,20 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     if (ok && busy) {
 #pragma unroll 1
       for (int h = 0; h < a.sgroups; ++h) {
-        const uint16_t* M = met + b * SG * 32 + h * kDG * 32 + lane;
-        const uint32_t* Wb = win + b * wbuf + h * kDG * cspan + lead + wd * KW;
+        const uint32_t* M = met + b * SG * 32 + h * kDG * 32 + lane;
+        const uint32_t Wb = smem_u32(win + b * wbuf + lead + wd * KW);
+        static_assert(KW == 2 || KW == 4, "window words per lane");
         auto fetch = [&](int ci, uint32_t (&v)[KW]) {
           const uint32_t m = M[ci * 32];
-          const uint32_t* p = Wb + ci * cspan + (m >> 5);
+          const uint32_t p = Wb + (m >> 5);
           uint32_t x[KW + 1];
-#pragma unroll
-          for (int j = 0; j <= KW; ++j) x[j] = p[j];
+          x[0] = lds32<0>(p);
+          x[1] = lds32<4>(p);
+          x[2] = lds32<8>(p);
+          if constexpr (KW == 4) {
+            x[3] = lds32<12>(p);
+            x[4] = lds32<16>(p);
+          }
 #pragma unroll
           for (int j = 0; j < KW; ++j) v[j] = __funnelshift_r(x[j], x[j + 1], m);
         };

@@ -268,14 +268,7 @@ cudaError_t run_z(const ZArgs& a, dim3 grid, dim3 block, int smem, cudaStream_t 
   return cudaGetLastError();
 }
 
-// 32-bit loads and stores at a shared-memory byte address plus a constant: one instruction each, where
-// a generic pointer costs its address arithmetic again for every unrolled slot
-template <int OFF>
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.b32 %0, [%1 + %2];" : "=r"(v) : "r"(addr), "n"(OFF));
-  return v;
-}
+// 32-bit store at a shared-memory byte address plus a constant (lds32's counterpart)
 template <int OFF>
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0 + %1], %2;" ::"r"(addr), "n"(OFF), "r"(v) : "memory");
