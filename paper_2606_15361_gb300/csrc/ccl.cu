@@ -15,6 +15,7 @@
 // Every data-dependent loop is bounded; a bound that is hit sets a status bit instead of
 // spinning.
 
+#include <algorithm>
 #include <vector>
 
 #include "snd_internal.h"
@@ -178,6 +179,7 @@ __device__ __forceinline__ void run_count_row(const uint32_t* __restrict__ m, in
   const int nbw = (nb + 31) >> 5;
   const uint32_t* row = m + static_cast<size_t>(warp) * mw;
   int cnt = 0;
+#pragma unroll 4
   for (int q0 = 0; q0 < nbw; q0 += 32) {
     const int q = q0 + lane;
     const uint32_t w = q < nbw ? row[q] : 0u;
@@ -252,9 +254,12 @@ __device__ __forceinline__ void run_write_row(const uint32_t* __restrict__ m, in
   const int nbw = (nb + 31) >> 5;
   const uint32_t* row = m + static_cast<size_t>(warp) * mw;
   int base_s = row_runs[warp], base_e = row_runs[warp];
+  uint32_t ahead = lane < nbw ? row[lane] : 0u;  // the next 32 words, loaded one round early
   for (int q0 = 0; q0 < nbw; q0 += 32) {
     const int q = q0 + lane;
-    const uint32_t w = q < nbw ? row[q] : 0u;
+    const uint32_t w = ahead;
+    ahead = q + 32 < nbw ? row[q + 32] : 0u;
+    if (!__any_sync(0xFFFFFFFFu, w != 0u)) continue;  // no run starts or ends here
     const uint32_t prev = (q > 0 && q - 1 < nbw) ? row[q - 1] : 0u;
     const uint32_t next = (q + 1 < nbw) ? row[q + 1] : 0u;
     uint32_t st = w & ~((w << 1) | (prev >> 31));
@@ -406,7 +411,14 @@ __device__ __forceinline__ void peak_items(const MfCell* cells, uint32_t* counte
     const unsigned long long key =
         (static_cast<unsigned long long>(__float_as_uint(c.snr)) << 32) | (0xFFFFFFFFull - c.cell);
     if (pass == 0) {
-      atomicMax(&peak[root], key);
+      // one atomic per island among the warp's lanes here (cells next to each other in the list mostly
+      // share an island, and its one address would take them one after the other). S/N bits order as
+      // the S/N does, as all are positive.
+      const unsigned lanes = __match_any_sync(__activemask(), root);
+      const unsigned hi = __reduce_max_sync(lanes, static_cast<unsigned>(key >> 32));
+      const unsigned lo = __reduce_max_sync(lanes, (key >> 32) == hi ? static_cast<unsigned>(key) : 0u);
+      if ((threadIdx.x & 31) == __ffs(lanes) - 1)
+        atomicMax(&peak[root], (static_cast<unsigned long long>(hi) << 32) | lo);
     } else if (peak[root] == key) {
       pwidth[root] = c.width;
     }
@@ -492,7 +504,7 @@ __device__ __forceinline__ void bump(uint32_t* counters, int cand_cap) {
 __global__ void k_bump(uint32_t* counters, int cand_cap) { bump(counters, cand_cap); }
 
 // ---------------------------------------------------------------------------------------
-// Candidate stage of many plans in ONE cooperative launch: the stages above run one after
+// Candidate stage of one or many plans in ONE cooperative launch: the stages above run one after
 // another over all beams' blocks, separated by grid-wide barriers (every CTA is resident, as a
 // cooperative launch guarantees). Each barrier is a counter + generation pair in device
 // memory; its wait is bounded, and a wait that runs out marks every beam's status word and
@@ -533,24 +545,36 @@ __device__ __forceinline__ int cbeam_of(const int* first, int n, int i) {
   return lo;
 }
 
-__device__ bool grid_barrier(const CandMulti& m) {
+// Grid-wide barrier; the CTA that arrives last runs `last` before it lets the others go on.
+template <typename F>
+__device__ __forceinline__ bool grid_barrier(const CandMulti& m, F&& last) {
+  __shared__ int s_last;
+  __shared__ unsigned int s_gen;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_gen = *static_cast<volatile unsigned int*>(m.gbar + 1);
+    __threadfence();
+    s_last = atomicAdd(m.gbar, 1u) == gridDim.x - 1;
+  }
   __syncthreads();
   int ok = 1;
-  if (threadIdx.x == 0) {
-    volatile unsigned int* gen = m.gbar + 1;
-    const unsigned int g = *gen;
+  if (s_last) {
     __threadfence();
-    if (atomicAdd(m.gbar, 1u) == gridDim.x - 1) {
+    last();
+    __syncthreads();
+    if (threadIdx.x == 0) {
       m.gbar[0] = 0;
       __threadfence();
       atomicAdd(m.gbar + 1, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*gen == g) {
-        if (clock64() - t0 > m.wait_cycles) {
-          ok = 0;
-          break;
-        }
+    }
+  } else if (threadIdx.x == 0) {
+    volatile unsigned int* gen = m.gbar + 1;
+    const unsigned int g = s_gen;
+    const long long t0 = clock64();
+    while (*gen == g) {
+      if (clock64() - t0 > m.wait_cycles) {
+        ok = 0;
+        break;
       }
     }
     __threadfence();
@@ -559,12 +583,61 @@ __device__ bool grid_barrier(const CandMulti& m) {
   }
   return __syncthreads_and(ok) != 0;
 }
+__device__ __forceinline__ bool grid_barrier(const CandMulti& m) { return grid_barrier(m, [] {}); }
 
+// Whether this CTA is the last to get here (a barrier that nobody waits at).
+__device__ __forceinline__ bool grid_last(const CandMulti& m) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(m.gbar, 1u) == gridDim.x - 1;
+    if (s_last) m.gbar[0] = 0;
+  }
+  __syncthreads();
+  if (s_last) __threadfence();
+  return s_last != 0;
+}
+
+// A block of at most this many runs (the usual block has a few hundred) has its islands joined by one
+// CTA in shared memory: a root walk there takes tens of cycles a step, in global memory hundreds.
+constexpr int kSmallRuns = 2048;
+
+__device__ __forceinline__ void join_small(const CandBeam& e, int n, uint32_t* csm) {
+  int* par = reinterpret_cast<int*>(csm);
+  int *pix = par + kSmallRuns, *st = pix + kSmallRuns, *en = st + kSmallRuns;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < n; i += 256) {
+    par[i] = i;
+    pix[i] = 0;
+    st[i] = e.run_start[i];
+    en[i] = e.run_end[i];
+  }
+  __syncthreads();
+  union_items(e.row_runs, e.ndm, e.run_cap, st, en, e.run_row, par, e.counters, e.lim, tid, 256);
+  __syncthreads();
+  flatten_items(e.row_runs, e.ndm, e.run_cap, st, en, par, pix, e.counters, e.lim, tid, 256);
+  __syncthreads();
+  for (int i = tid; i < n; i += 256) {
+    e.parent[i] = par[i];
+    e.npix[i] = pix[i];
+  }
+}
+
+// What bounds it is latency: a few hundred runs and some ten thousand cells per block go through nine
+// dependent steps. So the grid is no larger than the block's tiles and rows need, one plan's short
+// serial steps (the scan, joining a small block's islands, the final list) run in the CTA that a barrier
+// saw last, and the cells' peaks are reduced in the warp before their atomics. Stage times before and
+// after, us with the event pair (before: ten barriers of 304 CTAs and global walks): 128 x 1024 binary
+// 38 -> 29, 128 x 16384 65 -> 50, 2048 x 16384 binary 56 -> 48, graded 113 -> 66, float 81 -> 57; eight
+// beams (one launch) 517 -> 315.
 __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ CandMulti m) {
   extern __shared__ uint32_t csm[];
   const int nblk = gridDim.x, bid = blockIdx.x, tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int gtid = bid * 256 + tid, gthreads = nblk * 256;
+  const bool one = m.nbeams == 1;  // one plan: its serial steps run inside the barriers
+  const CandBeam& e0 = m.beam[0];
   // 1. closing (a plain copy for a 1 x 1 element)
   for (int v = bid; v < m.total_close; v += nblk) {
     const int b = cbeam_of(m.first_close, m.nbeams, v);
@@ -584,49 +657,84 @@ __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ Cand
     __syncthreads();
   }
   if (!grid_barrier(m)) return;
-  // 2. runs per row
+  // 2. runs per row, 3. scan of the run counts (many plans: one CTA per beam)
   for (int v = bid; v < m.total_rows; v += nblk) {
     const int b = cbeam_of(m.first_rows, m.nbeams, v);
     const CandBeam& e = m.beam[b];
     run_count_row(e.mask3, e.ndm, e.mw, e.nb, e.row_runs, (v - m.first_rows[b]) * 8 + warp, lane);
   }
-  if (!grid_barrier(m)) return;
-  // 3. scan of the run counts, one CTA per beam
-  for (int b = bid; b < m.nbeams; b += nblk) {
-    const CandBeam& e = m.beam[b];
-    scan_rows_cta<256>(e.row_runs, e.ndm, e.counters, e.run_cap);
-    __syncthreads();
+  if (!grid_barrier(m, [&] {
+        if (one) scan_rows_cta<256>(e0.row_runs, e0.ndm, e0.counters, e0.run_cap);
+      }))
+    return;
+  if (!one) {
+    for (int b = bid; b < m.nbeams; b += nblk) {
+      const CandBeam& e = m.beam[b];
+      scan_rows_cta<256>(e.row_runs, e.ndm, e.counters, e.run_cap);
+      __syncthreads();
+    }
+    if (!grid_barrier(m)) return;
   }
-  if (!grid_barrier(m)) return;
-  // 4. runs and union-find state
+  // 4. runs and union-find state, then the islands of small blocks (many plans: one CTA per beam)
   for (int v = bid; v < m.total_rows; v += nblk) {
     const int b = cbeam_of(m.first_rows, m.nbeams, v);
     const CandBeam& e = m.beam[b];
     run_write_row(e.mask3, e.ndm, e.mw, e.nb, e.row_runs, e.run_start, e.run_end, e.run_row, e.parent, e.npix,
                   e.peak, e.pwidth, e.run_cap, (v - m.first_rows[b]) * 8 + warp, lane);
   }
-  if (!grid_barrier(m)) return;
-  // 5. - 10. over each beam's runs, cells and block candidates
-  for (int b = 0; b < m.nbeams; ++b) {
-    const CandBeam& e = m.beam[b];
-    union_items(e.row_runs, e.ndm, e.run_cap, e.run_start, e.run_end, e.run_row, e.parent, e.counters, e.lim, gtid,
-                gthreads);
+  auto runs_of = [&](const CandBeam& e) { return runs_total(e.row_runs, e.ndm, e.run_cap); };
+  if (!grid_barrier(m, [&] {
+        const int n = one ? runs_of(e0) : 0;
+        if (one && n >= 0 && n <= kSmallRuns) join_small(e0, n, csm);
+      }))
+    return;
+  bool large = false;  // a block whose runs the whole grid joins
+  for (int b = 0; b < m.nbeams; ++b) large = large || runs_of(m.beam[b]) > kSmallRuns;
+  if (!one || large) {
+    if (!one)
+      for (int b = bid; b < m.nbeams; b += nblk) {
+        const int n = runs_of(m.beam[b]);
+        if (n >= 0 && n <= kSmallRuns) join_small(m.beam[b], n, csm);
+        __syncthreads();
+      }
+    for (int b = 0; b < m.nbeams; ++b) {
+      const CandBeam& e = m.beam[b];
+      if (runs_of(e) > kSmallRuns)
+        union_items(e.row_runs, e.ndm, e.run_cap, e.run_start, e.run_end, e.run_row, e.parent, e.counters, e.lim, gtid,
+                    gthreads);
+    }
+    if (!grid_barrier(m)) return;
   }
-  if (!grid_barrier(m)) return;
-  for (int b = 0; b < m.nbeams; ++b) {
-    const CandBeam& e = m.beam[b];
-    flatten_items(e.row_runs, e.ndm, e.run_cap, e.run_start, e.run_end, e.parent, e.npix, e.counters, e.lim, gtid,
-                  gthreads);
+  if (large) {
+    for (int b = 0; b < m.nbeams; ++b) {
+      const CandBeam& e = m.beam[b];
+      if (runs_of(e) > kSmallRuns)
+        flatten_items(e.row_runs, e.ndm, e.run_cap, e.run_start, e.run_end, e.parent, e.npix, e.counters, e.lim, gtid,
+                      gthreads);
+    }
+    if (!grid_barrier(m)) return;
   }
-  if (!grid_barrier(m)) return;
+  // 5. peaks: every cell, twice
   for (int pass = 0; pass < 2; ++pass) {
     for (int b = 0; b < m.nbeams; ++b) {
       const CandBeam& e = m.beam[b];
       peak_items(e.cells, e.counters, e.cell_cap, e.nb, e.row_runs, e.ndm, e.run_cap, e.run_start, e.run_end,
                  e.parent, e.peak, e.pwidth, pass, gtid, gthreads);
     }
-    if (!grid_barrier(m)) return;
+    if (pass == 0 && !grid_barrier(m)) return;
   }
+  // 6. the block's candidates, ranked and appended
+  if (one && !large) {
+    if (!grid_last(m)) return;
+    emit_items(e0.row_runs, e0.ndm, e0.run_cap, e0.parent, e0.npix, e0.peak, e0.pwidth, e0.nb, e0.n_min, e0.f_prev,
+               e0.dm_f32, e0.bcand, e0.cand_cap, e0.counters, tid, 256);
+    __syncthreads();
+    rank_items(e0.bcand, e0.cand, e0.counters, e0.cand_cap, tid, 256);
+    __syncthreads();
+    if (tid == 0) bump(e0.counters, e0.cand_cap);
+    return;
+  }
+  if (!grid_barrier(m)) return;
   for (int b = 0; b < m.nbeams; ++b) {
     const CandBeam& e = m.beam[b];
     emit_items(e.row_runs, e.ndm, e.run_cap, e.parent, e.npix, e.peak, e.pwidth, e.nb, e.n_min, e.f_prev, e.dm_f32,
@@ -759,7 +867,7 @@ cudaError_t launch_candidates_batch(const Plan* const* plans, const ChunkPos* po
     const Plan& owner = *plans[batch[i0]];
     m.gbar = owner.dp.counters + kCntGridBar;
     m.wait_cycles = owner.wait_limit > 0 ? owner.wait_limit : kGridWaitCycles;
-    const int smem = 2 * (kCloseTR + 4 * rmax) * kCloseNQ * static_cast<int>(sizeof(uint32_t));
+    const int smem = std::max(2 * (kCloseTR + 4 * rmax) * kCloseNQ, 4 * kSmallRuns) * static_cast<int>(sizeof(uint32_t));
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -768,8 +876,9 @@ cudaError_t launch_candidates_batch(const Plan* const* plans, const ChunkPos* po
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     if (e == cudaSuccess) e = cudaMemsetAsync(m.gbar, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    // one CTA per SM at most 2: the stages are latency bound, and fewer CTAs make cheaper barriers
-    const int grid = nsm * (per_sm < 2 ? per_sm : 2);
+    // at most two CTAs per SM, and no more than there are tiles or row groups (a few at least, for the
+    // cells): the stages are latency bound, and fewer CTAs make cheaper barriers
+    const int grid = std::min(nsm * std::min(per_sm, 2), std::max(16, std::max(m.total_close, m.total_rows)));
     void* args[] = {&m};
     e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_cand_multi), dim3(grid), dim3(256), args,
                                     static_cast<size_t>(smem), s);
