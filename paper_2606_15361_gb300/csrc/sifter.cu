@@ -98,10 +98,12 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
+// The last operand lets the hardware suspend the warp for up to 10 ms: without it the polling of a dozen
+// waiting warps took two thirds of the instructions that the convolutions' warps issued.
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x989680;\n selp.u32 %0, 1, 0, p;\n}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
       : "memory");
@@ -188,6 +190,39 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 16 consecutive TMEM columns at each of two addresses (one wait for both)
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float* va, float* vb) {
+  uint32_t r[16], q[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(ta));
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]), "=r"(q[8]),
+        "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+      : "r"(tb));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    va[i] = __uint_as_float(r[i]);
+    vb[i] = __uint_as_float(q[i]);
+  }
+}
+
+// The 2x2 max pooling of 16 channels (inference). Lanes x even, x odd hold the two columns of a pooled
+// cell, v0 / v1 the lane's two rows. The even lane ends with channels 0 .. 7 of the cell, the odd lane
+// with 8 .. 15, so a value is exchanged per channel pair and both lanes store.
+__device__ __forceinline__ void pool_half16(const float* v0, const float* v1, int lane, float* out) {
+  const bool odd = lane & 1;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float a = fmaxf(v0[q], v1[q]), b = fmaxf(v0[q + 8], v1[q + 8]);
+    out[q] = fmaxf(odd ? b : a, __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1));
+  }
 }
 
 // BF16 of relu(v + bias), two values packed
@@ -478,7 +513,7 @@ __global__ void __launch_bounds__(320, 2)
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ float bsm[COUT];
-  uint8_t* hsm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(hsm_raw) + 127) & ~uintptr_t(127));
+  uint8_t* hsm = hsm_raw + (-smem_u32(hsm_raw) & 127u);
   const uint32_t sX = smem_u32(hsm), sW = sX + S * SB;
   bf16* wsm = reinterpret_cast<bf16*>(hsm + S * SB);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -618,38 +653,40 @@ __global__ void __launch_bounds__(320, 2)
 #pragma unroll 1
         for (int c = 0; c < COUT; c += 16) {
           float v0[16], v1[16];
-          tmem_ld16(tmem + lanes + static_cast<uint32_t>((bb * T) * COUT + c), v0);
-          tmem_ld16(tmem + lanes + static_cast<uint32_t>((bb * T + 1) * COUT + c), v1);
-          uint32_t pk[8];
+          tmem_ld16x2(tmem + lanes + static_cast<uint32_t>((bb * T) * COUT + c),
+                      tmem + lanes + static_cast<uint32_t>((bb * T + 1) * COUT + c), v0, v1);
+          const long long pix = (static_cast<long long>(b) * h2 + yp) * w2 + x2;
+          bf16* rows = a.p + static_cast<long long>(b) * COUT * h2 * w2 + static_cast<long long>(yp) * w2 + x2;
           if constexpr (TRAIN) {
             // training: the four rounded activations and their argmax (first maximum)
-            pool_argmax16(v0, v1, bsm + c, lane, pk, a.am, c, static_cast<long long>(a.n) * h2 * w2,
-                          (static_cast<long long>(b) * h2 + yp) * w2 + x2);
-          } else {
+            uint32_t pk[8];
+            pool_argmax16(v0, v1, bsm + c, lane, pk, a.am, c, static_cast<long long>(a.n) * h2 * w2, pix);
+            if (!(lane & 1)) {
+              if (a.pool_cl) {  // channels-last [(b, y2, x2)][COUT]
+                uint4* dst = reinterpret_cast<uint4*>(a.p + pix * COUT + c);
+                dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+              } else {  // fc1's rows [b][(c, y2, x2)]
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              const float m = fmaxf(v0[q], v1[q]);
-              v0[q] = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-            }
-          }
-          if (!(lane & 1)) {
-            if constexpr (!TRAIN) {
-#pragma unroll
-              for (int q = 0; q < 16; q += 2) pk[q >> 1] = act_pack2(v0[q], bsm[c + q], v0[q + 1], bsm[c + q + 1]);
-            }
-            if (a.pool_cl) {  // channels-last [(b, y2, x2)][COUT]
-              uint4* dst = reinterpret_cast<uint4*>(a.p + ((static_cast<long long>(b) * h2 + yp) * w2 + x2) * COUT + c);
-              dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-            } else {  // fc1's rows [b][(c, y2, x2)]
-              bf16* dst = a.p + static_cast<long long>(b) * COUT * h2 * w2 + static_cast<long long>(yp) * w2 + x2;
-#pragma unroll
-              for (int q = 0; q < 16; ++q) {
-                const bf16 v = __ushort_as_bfloat16(
-                    static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
-                dst[static_cast<long long>(c + q) * h2 * w2] = v;
-
+                for (int q = 0; q < 16; ++q)
+                  rows[static_cast<long long>(c + q) * h2 * w2] = __ushort_as_bfloat16(
+                      static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
               }
+            }
+          } else {
+            float m[8];
+            pool_half16(v0, v1, lane, m);
+            const int ch = c + 8 * (lane & 1);  // this lane's first channel
+            uint32_t pk[4];
+#pragma unroll
+            for (int q = 0; q < 8; q += 2) pk[q >> 1] = act_pack2(m[q], bsm[ch + q], m[q + 1], bsm[ch + q + 1]);
+            if (a.pool_cl) {
+              *reinterpret_cast<uint4*>(a.p + pix * COUT + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                rows[static_cast<long long>(ch + q) * h2 * w2] = __ushort_as_bfloat16(
+                    static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
             }
           }
         }
@@ -677,12 +714,13 @@ __global__ void __launch_bounds__(320, 2)
 // reads the next row or a zero row): two MMAs of K = 16 per tile, weights [ky][cout][8] with
 // zeros past kx = 2 and ky = 2.
 // The epilogue writes the 2x2 max pooling of the activations, channels-last [(b, y2, x2)][16];
-// TRAIN: also the argmax of every pooled cell (am). 320 threads: warps 0-3 epilogue,
-// warps 4-7 build U, warp 8 owns TMEM and issues the MMAs, warp 9 issues the TMA loads.
+// TRAIN: also the argmax of every pooled cell (am). 448 threads: two epilogue warpgroups (warps 0-3
+// and 4-7), each draining one of the two TMEM accumulator buffers, warps 8-11 build U, warp 12 owns
+// TMEM and issues the MMAs, warp 13 issues the TMA loads.
 // Rounding: BF16 snippet values and weights, FP32 sums (the tensor core adds the nine
 // products in its own order), bias, ReLU, BF16 store.
 template <bool TRAIN>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(448, TRAIN ? 2 : 3)
     k_conv1_tc(const __grid_constant__ CUtensorMap mx, int n, const float* __restrict__ w, const float* __restrict__ bias,
                bf16* __restrict__ out, uint32_t* __restrict__ am, uint32_t* err) {
   constexpr int RS = 12, US = 4;               // raw and U stages
@@ -697,7 +735,7 @@ __global__ void __launch_bounds__(320, 1)
   __shared__ float bsm[16];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  uint8_t* csm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(csm_raw) + 127) & ~uintptr_t(127));
+  uint8_t* csm = csm_raw + (-smem_u32(csm_raw) & 127u);  // an offset, so that it stays a shared address
   const uint32_t sU = smem_u32(csm), sR = sU + US * UB;
   const float* raw = reinterpret_cast<const float*>(csm + US * UB);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -728,7 +766,7 @@ __global__ void __launch_bounds__(320, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 8) {
+  if (warp == 12) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(kCols)
                  : "memory");
@@ -740,7 +778,7 @@ __global__ void __launch_bounds__(320, 1)
   const uint32_t tmem = tmem_slot;
   volatile int* abort_v = &abort_flag;
 
-  if (warp == 9) {
+  if (warp == 13) {
     if (lane == 0) {
       int j = 0;
       for (int it = blockIdx.x; it < items && !*abort_v; it += gridDim.x, ++j) {
@@ -756,8 +794,8 @@ __global__ void __launch_bounds__(320, 1)
         tma_load_2d_rows(sR + r * RB, &mx, rb, hx * 128 - 4, 2 * yp - 1, b);
       }
     }
-  } else if (warp >= 4 && warp < 8) {
-    const int pr = threadIdx.x - 128;  // pixel of the half row
+  } else if (warp >= 8 && warp < 12) {
+    const int pr = threadIdx.x - 256;  // pixel of the half row
     int j = 0;
     for (int it = blockIdx.x; it < items && !*abort_v; it += gridDim.x, ++j) {
       const int r = j % RS, u = j % US;
@@ -788,7 +826,7 @@ __global__ void __launch_bounds__(320, 1)
         mbar_arrive(smem_u32(&bar_u[u]));
       }
     }
-  } else if (warp == 8) {
+  } else if (warp == 12) {
     if (lane == 0) {
       constexpr uint32_t idesc = mma_idesc(16);
       int j = 0;
@@ -821,10 +859,11 @@ __global__ void __launch_bounds__(320, 1)
       }
     }
   } else {
-    // epilogue warps 0-3 (TMEM lanes 32 warp ..: pixel 32 warp + lane of the half row)
-    int j = 0;
-    for (int it = blockIdx.x; it < items; it += gridDim.x, ++j) {
-      const int bb = j & 1;
+    // epilogue warpgroup grp (warps 4 grp ..): the items j with j & 1 == grp, from TMEM buffer grp;
+    // warp wq of the group reads TMEM lanes 32 wq .. (pixel 32 wq + lane of the half row)
+    const int bb = warp >> 2, wq = warp & 3;
+    int j = bb;
+    for (int it = blockIdx.x + bb * gridDim.x; it < items; it += 2 * gridDim.x, j += 2) {
       bool ok = !*abort_v && mbar_wait(smem_u32(&bar_tfull[bb]), (j >> 1) & 1);
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (!ok) {
@@ -833,36 +872,32 @@ __global__ void __launch_bounds__(320, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t lanes = static_cast<uint32_t>(warp * 32) << 16;
+      const uint32_t lanes = static_cast<uint32_t>(wq * 32) << 16;
       const int b = it >> 6, yp = (it >> 1) & 31, hx = it & 1;
-      const int xg = hx * 128 + warp * 32 + lane;
+      const int xg = hx * 128 + wq * 32 + lane;
+      const long long pix = (static_cast<long long>(b) * 32 + yp) * 128 + (xg >> 1);
       float v0[16], v1[16];
-      tmem_ld16(tmem + lanes + static_cast<uint32_t>((bb * 2) * 16), v0);
-      tmem_ld16(tmem + lanes + static_cast<uint32_t>((bb * 2 + 1) * 16), v1);
-      {
+      tmem_ld16x2(tmem + lanes + static_cast<uint32_t>((bb * 2) * 16), tmem + lanes + static_cast<uint32_t>((bb * 2 + 1) * 16),
+                  v0, v1);
+      if constexpr (TRAIN) {
+        // training: the four rounded activations and their argmax (first maximum)
         uint32_t pk[8];
-        if constexpr (TRAIN) {
-          // training: the four rounded activations and their argmax (first maximum)
-          pool_argmax16(v0, v1, bsm, lane, pk, am, 0, static_cast<long long>(n) * 32 * 128,
-                        (static_cast<long long>(b) * 32 + yp) * 128 + (xg >> 1));
-        } else {
-          // the maximum of the four rounded activations is the rounded activation of the
-          // largest of the four sums (bias, ReLU and BF16 rounding are monotone non-decreasing)
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            const float m = fmaxf(v0[q], v1[q]);
-            v0[q] = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-          }
-        }
+        pool_argmax16(v0, v1, bsm, lane, pk, am, 0, static_cast<long long>(n) * 32 * 128, pix);
         if (!(lane & 1)) {
-          if constexpr (!TRAIN) {
-#pragma unroll
-            for (int q = 0; q < 16; q += 2) pk[q >> 1] = act_pack2(v0[q], bsm[q], v0[q + 1], bsm[q + 1]);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(out + ((static_cast<long long>(b) * 32 + yp) * 128 + (xg >> 1)) * 16);
+          uint4* dst = reinterpret_cast<uint4*>(out + pix * 16);
           dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
         }
+      } else {
+        // the maximum of the four rounded activations is the rounded activation of the
+        // largest of the four sums (bias, ReLU and BF16 rounding are monotone non-decreasing)
+        float m[8];
+        pool_half16(v0, v1, lane, m);
+        const int ch = 8 * (lane & 1);  // this lane's first channel
+        uint32_t pk[4];
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) pk[q >> 1] = act_pack2(m[q], bsm[ch + q], m[q + 1], bsm[ch + q + 1]);
+        *reinterpret_cast<uint4*>(out + pix * 16 + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -872,7 +907,7 @@ __global__ void __launch_bounds__(320, 1)
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 8) {
+  if (warp == 12) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
   }
 }
@@ -1596,9 +1631,9 @@ int conv1_tc(const float* x, int n, const float* w, const float* bias, bf16* out
   const int items = n * 64;
   auto go = [&](auto kern) {
     int grid = 0;
-    const cudaError_t e = persistent_grid(kern, smem, 320, 64, items, &grid);
+    const cudaError_t e = persistent_grid(kern, smem, 448, 64, items, &grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, 320, smem, s>>>(mx, n, w, bias, out, am, err);
+    kern<<<grid, 448, smem, s>>>(mx, n, w, bias, out, am, err);
     return cudaGetLastError();
   };
   const cudaError_t e = am ? go(k_conv1_tc<true>) : go(k_conv1_tc<false>);
