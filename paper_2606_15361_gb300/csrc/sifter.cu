@@ -427,32 +427,39 @@ struct ConvArgs {
 // the gradient to the argmax). Lane pairs (x even, x odd) hold one pooled cell; v0 / v1 are the
 // FP32 sums of the lane's pixel in the upper / lower row. Each activation is bias, ReLU and
 // BF16 rounding of its sum; the cell takes the first maximum in row-major order (upper left,
-// upper right, lower left, lower right), as the oracle's pooling does. Even lanes get the packed pooled
-// values in pk and write the 16 argmaxes, 2 bits each (channel c0 + q at bits 2q, 2q + 1), as one
-// word am[(c0 / 16) * npix + pix].
+// upper right, lower left, lower right), as the oracle's pooling does. The even lane ends with
+// channels 0 .. 7 of the cell, the odd lane with 8 .. 15 (a channel's two rows cross in one
+// exchange as a BF16 pair): the packed pooled values in pk, the argmaxes, 2 bits each, as its half
+// of the word am[(c0 / 16) * npix + pix] (channel c0 + q at bits 2q, 2q + 1).
 __device__ __forceinline__ void pool_argmax16(const float* v0, const float* v1, const float* bias, int lane,
                                               uint32_t* pk, uint32_t* am, int c0, long long npix, long long pix) {
+  const bool odd = lane & 1;
   uint32_t code = 0;
 #pragma unroll
-  for (int q = 0; q < 16; q += 2) {
+  for (int q = 0; q < 8; q += 2) {
     float best[2];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const float u = __bfloat162float(__float2bfloat16_rn(fmaxf(v0[q + e] + bias[q + e], 0.0f)));
-      const float l = __bfloat162float(__float2bfloat16_rn(fmaxf(v1[q + e] + bias[q + e], 0.0f)));
-      const float ur = __shfl_xor_sync(0xFFFFFFFFu, u, 1), lr = __shfl_xor_sync(0xFFFFFFFFu, l, 1);
+      const int k = q + e;
+      // (upper, lower) of channel k and of channel k + 8 in this lane's column
+      const uint32_t lo = act_pack2(v0[k], bias[k], v1[k], bias[k]);
+      const uint32_t hi = act_pack2(v0[k + 8], bias[k + 8], v1[k + 8], bias[k + 8]);
+      const uint32_t own = odd ? hi : lo, got = __shfl_xor_sync(0xFFFFFFFFu, odd ? lo : hi, 1);
+      const uint32_t left = odd ? got : own, right = odd ? own : got;
+      const float ul = __uint_as_float(left << 16), ll = __uint_as_float(left & 0xFFFF0000u);
+      const float ur = __uint_as_float(right << 16), lr = __uint_as_float(right & 0xFFFF0000u);
       int a = 0;
-      float bv = u;
+      float bv = ul;
       if (ur > bv) { bv = ur; a = 1; }
-      if (l > bv) { bv = l; a = 2; }
+      if (ll > bv) { bv = ll; a = 2; }
       if (lr > bv) { bv = lr; a = 3; }
       best[e] = bv;
-      code |= static_cast<uint32_t>(a) << (2 * (q + e));
+      code |= static_cast<uint32_t>(a) << (2 * k);
     }
     const __nv_bfloat162 pr = __floats2bfloat162_rn(best[0], best[1]);
     pk[q >> 1] = *reinterpret_cast<const uint32_t*>(&pr);
   }
-  if (!(lane & 1)) am[static_cast<long long>(c0 >> 4) * npix + pix] = code;
+  reinterpret_cast<uint16_t*>(am + static_cast<long long>(c0 >> 4) * npix + pix)[lane & 1] = static_cast<uint16_t>(code);
 }
 
 // ---------------------------------------------------------------- halo convolution
@@ -657,37 +664,24 @@ __global__ void __launch_bounds__(320, 2)
                       tmem + lanes + static_cast<uint32_t>((bb * T + 1) * COUT + c), v0, v1);
           const long long pix = (static_cast<long long>(b) * h2 + yp) * w2 + x2;
           bf16* rows = a.p + static_cast<long long>(b) * COUT * h2 * w2 + static_cast<long long>(yp) * w2 + x2;
+          const int ch = c + 8 * (lane & 1);  // this lane's first channel
+          uint32_t pk[4];
           if constexpr (TRAIN) {
             // training: the four rounded activations and their argmax (first maximum)
-            uint32_t pk[8];
             pool_argmax16(v0, v1, bsm + c, lane, pk, a.am, c, static_cast<long long>(a.n) * h2 * w2, pix);
-            if (!(lane & 1)) {
-              if (a.pool_cl) {  // channels-last [(b, y2, x2)][COUT]
-                uint4* dst = reinterpret_cast<uint4*>(a.p + pix * COUT + c);
-                dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-              } else {  // fc1's rows [b][(c, y2, x2)]
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                  rows[static_cast<long long>(c + q) * h2 * w2] = __ushort_as_bfloat16(
-                      static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
-              }
-            }
           } else {
             float m[8];
             pool_half16(v0, v1, lane, m);
-            const int ch = c + 8 * (lane & 1);  // this lane's first channel
-            uint32_t pk[4];
 #pragma unroll
             for (int q = 0; q < 8; q += 2) pk[q >> 1] = act_pack2(m[q], bsm[ch + q], m[q + 1], bsm[ch + q + 1]);
-            if (a.pool_cl) {
-              *reinterpret_cast<uint4*>(a.p + pix * COUT + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            } else {
+          }
+          if (a.pool_cl) {  // channels-last [(b, y2, x2)][COUT]
+            *reinterpret_cast<uint4*>(a.p + pix * COUT + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          } else {  // fc1's rows [b][(c, y2, x2)]
 #pragma unroll
-              for (int q = 0; q < 8; ++q)
-                rows[static_cast<long long>(ch + q) * h2 * w2] = __ushort_as_bfloat16(
-                    static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
-            }
+            for (int q = 0; q < 8; ++q)
+              rows[static_cast<long long>(ch + q) * h2 * w2] = __ushort_as_bfloat16(
+                  static_cast<unsigned short>((q & 1) ? (pk[q >> 1] >> 16) : (pk[q >> 1] & 0xFFFFu)));
           }
         }
       }
@@ -879,26 +873,20 @@ __global__ void __launch_bounds__(448, TRAIN ? 2 : 3)
       float v0[16], v1[16];
       tmem_ld16x2(tmem + lanes + static_cast<uint32_t>((bb * 2) * 16), tmem + lanes + static_cast<uint32_t>((bb * 2 + 1) * 16),
                   v0, v1);
+      const int ch = 8 * (lane & 1);  // this lane's first channel
+      uint32_t pk[4];
       if constexpr (TRAIN) {
         // training: the four rounded activations and their argmax (first maximum)
-        uint32_t pk[8];
         pool_argmax16(v0, v1, bsm, lane, pk, am, 0, static_cast<long long>(n) * 32 * 128, pix);
-        if (!(lane & 1)) {
-          uint4* dst = reinterpret_cast<uint4*>(out + pix * 16);
-          dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        }
       } else {
         // the maximum of the four rounded activations is the rounded activation of the
         // largest of the four sums (bias, ReLU and BF16 rounding are monotone non-decreasing)
         float m[8];
         pool_half16(v0, v1, lane, m);
-        const int ch = 8 * (lane & 1);  // this lane's first channel
-        uint32_t pk[4];
 #pragma unroll
         for (int q = 0; q < 8; q += 2) pk[q >> 1] = act_pack2(m[q], bsm[ch + q], m[q + 1], bsm[ch + q + 1]);
-        *reinterpret_cast<uint4*>(out + pix * 16 + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
+      *reinterpret_cast<uint4*>(out + pix * 16 + ch) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_tempty[bb]));
