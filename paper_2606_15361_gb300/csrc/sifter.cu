@@ -902,89 +902,113 @@ __global__ void __launch_bounds__(448, TRAIN ? 2 : 3)
 
 // ---------------------------------------------------------------- layer kernels
 
-// conv1's weight gradient dW[co][tap] += sum over pixels m of dY^T[co][m] * x[m + tap offset]
-// (the snippet values rounded to BF16, as the forward convolution reads them; zero outside the
-// snippet). 16 x 9 outputs, so the CUDA cores reduce it directly: a CTA takes one snippet and 4
-// output channels (blockIdx.y) and stages the snippet in shared memory; a warp takes one image
-// row at a time (rows warp, warp + 8, ...), a lane 8 consecutive pixels, whose gradients come
-// as one 16-byte load per channel. A thread keeps its 36 partial sums in registers; the CTA's
-// sums are added atomically.
-__global__ void __launch_bounds__(256) k_dw1(const float* __restrict__ x, int n, const bf16* __restrict__ dyT,
-                                             float* __restrict__ dw) {
-  constexpr int XP = kW + 16;  // staged row (BF16): pixel xx at xx + 8, zero at 7 and kW + 8
-  __shared__ __align__(16) bf16 xs[kH + 2][XP];
-  __shared__ float red[8][36];
-  const int b = blockIdx.x, c0 = blockIdx.y * 4;
+// conv1's weight and bias gradients straight from the pooled gradient: dW[co][tap] += sum over pooled
+// cells of dP * x[argmax + tap offset] where the pooled activation is positive (the snippet values rounded
+// to BF16, as the forward convolution reads them; zero outside the snippet). Three of a cell's four pixels
+// get no gradient, so a cell and channel costs nine FMAs at its argmax, and the unpooled map (134 MB at
+// batch 256, written by one kernel and read by the next) is not made: 47 + 45 -> 43 us at batch 256.
+// What bounds it is the latency of the loads (a warp issues 46% of the time at four CTAs per SM; without
+// the loads ahead 57 us, eight steps ahead at three CTAs 53) and then the nine shared-memory loads a cell
+// and channel.
+// A CTA takes a quarter of a snippet, staged in FP32 with a border of one pixel; a warp takes one pooled row,
+// four cells at a time: lanes 8 q .. 8 q + 7 hold cell q's channel pairs, so gradients and activations are
+// one 128-byte row a load. The four cells' positions lie in two staged rows, whose pitch of 8 (mod 32) words
+// keeps them in different banks. A pixel that is not finite makes the taps that reach it NaN for every
+// channel, as the product with a zero gradient does.
+constexpr int kDw1Parts = 4;
+__global__ void __launch_bounds__(256, 4) k_dw1(const float* __restrict__ x, const bf16* __restrict__ dp,
+                                             const bf16* __restrict__ pooled, const uint32_t* __restrict__ am,
+                                             float* __restrict__ dw, float* __restrict__ db) {
+  constexpr int R = kH / kDw1Parts, XP = kW + 8;  // staged row: pixel xx at xx + 1
+  constexpr int W2 = kW / 2;
+  static_assert(kW == 256 && R / 2 == 8 && XP % 32 == 8, "one pixel a thread and row, one pooled row a warp");
+  __shared__ float xs[R + 2][XP];
+  __shared__ float red[8][16][10];
+  __shared__ unsigned bad;  // taps that reach a pixel that is not finite
+  const int b = blockIdx.x, y0 = blockIdx.y * R;
   const float* xb = x + static_cast<long long>(b) * kH * kW;
-  const int tx = threadIdx.x;
-  for (int r = 0; r < kH + 2; ++r) {
-    const int yy = r - 1;
-    xs[r][tx + 8] = __float2bfloat16_rn((yy >= 0 && yy < kH) ? xb[yy * kW + tx] : 0.0f);
-  }
-  if (tx < kH + 2) {
-    xs[tx][7] = __float2bfloat16_rn(0.0f);
-    xs[tx][kW + 8] = __float2bfloat16_rn(0.0f);
-  }
-  __syncthreads();
-  const long long mtot = static_cast<long long>(n) * kH * kW;
-  const int warp = tx >> 5, lane = tx & 31;
-  float acc[4][9];
+  const int tx = threadIdx.x, warp = tx >> 5, lane = tx & 31;
+  const int q = lane >> 3, c2 = lane & 7;
+  const int pix0 = (b * (kH / 2) + y0 / 2 + warp) * W2 + q;  // below 2^31 (the workspace is sized for it)
+  const uint32_t* gp = reinterpret_cast<const uint32_t*>(dp) + static_cast<long long>(pix0) * 8 + c2;
+  const uint32_t* pp = reinterpret_cast<const uint32_t*>(pooled) + static_cast<long long>(pix0) * 8 + c2;
+  const uint32_t* ap = am + pix0;
+  // four steps of gradients, activations and argmaxes, loaded while the four before them are summed (the
+  // first while the snippet is staged)
+  constexpr int kAhead = 4;
+  uint32_t gn[kAhead], pn[kAhead], an[kAhead];
+  auto load = [&](int i) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+    for (int u = 0; u < kAhead; ++u) {
+      gn[u] = gp[(i + u) * 32];
+      pn[u] = pp[(i + u) * 32];
+      an[u] = ap[(i + u) * 4];
+    }
+  };
+  load(0);
+  if (tx == 0) bad = 0u;
+  __syncthreads();
+#pragma unroll 9
+  for (int r = 0; r < R + 2; ++r) {
+    const int yy = y0 + r - 1;
+    const float v = __bfloat162float(__float2bfloat16_rn((yy >= 0 && yy < kH) ? xb[yy * kW + tx] : 0.0f));
+    xs[r][tx + 1] = v;
+    if (!isfinite(v)) {
+      unsigned m = 0u;
+      for (int k = 0; k < 9; ++k) {
+        const int y = yy - k / 3 + 1, xx = tx - k % 3 + 1;
+        if (y >= 0 && y < kH && xx >= 0 && xx < kW) m |= 1u << k;
+      }
+      atomicOr(&bad, m);
+    }
+  }
+  if (tx < 2 * (R + 2)) xs[tx >> 1][(tx & 1) ? kW + 1 : 0] = 0.0f;
+  __syncthreads();
+  const float* xr = &xs[2 * warp][2 * q];
+  float acc[2][9], bsum[2] = {0.0f, 0.0f};
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[j][k] = 0.0f;
-  const bf16* dyb = dyT + static_cast<long long>(c0) * mtot + static_cast<long long>(b) * kH * kW + 8 * lane;
-  // the gradients of the warp's next row are loaded while the current row is summed
-  uint4 gn[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) gn[j] = *reinterpret_cast<const uint4*>(dyb + j * mtot + warp * kW);
 #pragma unroll 1
-  for (int y = warp; y < kH; y += 8) {
-    uint4 gq[4];
+  for (int i = 0; i < W2 / 4; i += kAhead) {
+    uint32_t gw[kAhead], pw[kAhead], code[kAhead];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) gq[j] = gn[j];
-    if (y + 8 < kH) {
+    for (int u = 0; u < kAhead; ++u) gw[u] = gn[u], pw[u] = pn[u], code[u] = an[u] >> (4 * c2);
+    if (i + kAhead < W2 / 4) load(i + kAhead);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) gn[j] = *reinterpret_cast<const uint4*>(dyb + j * mtot + (y + 8) * kW);
-    }
+    for (int u = 0; u < kAhead; ++u)
 #pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-      // pixels 8 lane - 1 .. 8 lane + 8 of input row y + ky - 1 (staged row y + ky)
-      const bf16* row = &xs[y + ky][8 * lane + 8];
-      const uint4 mid = *reinterpret_cast<const uint4*>(row);
-      const bf16* mv = reinterpret_cast<const bf16*>(&mid);
-      float win[10];
-      win[0] = __bfloat162float(row[-1]);
+      for (int j = 0; j < 2; ++j) {
+        const float act = __uint_as_float(j ? pw[u] & 0xFFFF0000u : pw[u] << 16);
+        const float g = act > 0.0f ? __uint_as_float(j ? gw[u] & 0xFFFF0000u : gw[u] << 16) : 0.0f;
+        const float* at0 = xr + (i + u) * 8 + ((code[u] >> (2 * j + 1)) & 1u) * XP + ((code[u] >> (2 * j)) & 1u);
+        bsum[j] += g;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) win[k + 1] = __bfloat162float(mv[k]);
-      win[9] = __bfloat162float(row[8]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bf16* g = reinterpret_cast<const bf16*>(&gq[j]);
-#pragma unroll
-        for (int px = 0; px < 8; ++px) {
-          const float gv = __bfloat162float(g[px]);
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) acc[j][ky * 3 + kx] = fmaf(gv, win[px + kx], acc[j][ky * 3 + kx]);
-        }
+        for (int k = 0; k < 9; ++k) acc[j][k] = fmaf(g, at0[(k / 3) * XP + k % 3], acc[j][k]);
       }
-    }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      float v = acc[j][k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-      if (lane == 0) red[warp][j * 9 + k] = v;
+    for (int k = 0; k < 10; ++k) {
+      float v = k < 9 ? acc[j][k] : bsum[j];
+      v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
+      v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
+      if (q == 0) red[warp][2 * c2 + j][k] = v;
     }
   __syncthreads();
-  if (tx < 36) {
+  if (tx < 160) {
+    const int c = tx / 10, k = tx - 10 * c;
     float v = 0.0f;
 #pragma unroll
-    for (int w8 = 0; w8 < 8; ++w8) v += red[w8][tx];
-    atomicAdd(dw + c0 * 9 + tx, v);
+    for (int w8 = 0; w8 < 8; ++w8) v += red[w8][c][k];
+    if (k < 9) {
+      if ((bad >> k) & 1u) v = __int_as_float(0x7FC00000);
+      atomicAdd(dw + c * 9 + k, v);
+    } else {
+      atomicAdd(db + c, v);
+    }
   }
 }
 
@@ -1048,11 +1072,11 @@ __global__ void __launch_bounds__(256) k_transpose(const bf16* __restrict__ in, 
 // dP if its activation is positive, the other three positions zero. A thread owns one pooled
 // pixel and 16 channels c0 .. c0 + 15 (blockIdx.y), the lanes of a warp consecutive pixels of
 // one image row (w / 2 is a multiple of 32). CL: dP and the pooled map are channels-last BF16
-// [pix][CN] (conv1's and conv2's pooled maps, whose gradient the next layer's input-gradient
+// [pix][CN] (conv2's pooled map, whose gradient conv3's input-gradient
 // convolution writes), read as 16-byte vectors; else (conv3) dP is FP32 and the pooled map
 // BF16, both in fc1's row layout [b][(c, y2, x2)]. Writes dyT[c][m] as two 4-byte pairs per
-// channel (upper and lower row), coalesced along the row, and, when dy is set, the
-// channels-last dy[m][CN] of its four pixels as 16-byte stores. The bias gradient
+// channel (upper and lower row), coalesced along the row, and the channels-last dy[m][CN]
+// of its four pixels as 16-byte stores. The bias gradient
 // db[c] = sum over m of dY[c][m] (the BF16 values) is reduced over the CTA and added
 // atomically.
 template <int CN, bool CL>
@@ -1122,7 +1146,7 @@ __global__ void __launch_bounds__(256) k_unpool(const void* __restrict__ dpv, co
       d0[j >> 1] = e0; d1[j >> 1] = e1; d2[j >> 1] = e2; d3[j >> 1] = e3;
     }
   }
-  if (dy && valid) {
+  if (valid) {
     uint4* q0 = reinterpret_cast<uint4*>(dy + m00 * CN + c0);
     uint4* q1 = reinterpret_cast<uint4*>(dy + (m00 + 1) * CN + c0);
     uint4* q2 = reinterpret_cast<uint4*>(dy + (m00 + w) * CN + c0);
@@ -1680,7 +1704,7 @@ void layout(Sifter& f) {
     f.o.am[l] = take(4ull * (c.cout / 16) * (m / 4));
     if (f.training) {
       f.o.dy[l] = take(l > 0 ? 2ull * m * c.cout : 0);
-      f.o.dyT[l] = take(2ull * c.cout * m);
+      f.o.dyT[l] = take(l > 0 ? 2ull * c.cout * m : 0);
       f.o.s3[l] = take(l > 0 ? 2ull * 3 * c.cin * m : 0);  // the shifted copies of the layer's input
       f.o.dp[l] = take(l < 2 ? 2ull * c.cout * m / 4 : 0);
     }
@@ -1809,17 +1833,20 @@ int backward(Sifter& f, const float* x, const float* y, int n, cudaStream_t s) {
   for (int l = 2; l >= 0; --l) {
     const ConvL& c = kConv[l];
     const long long m = 1LL * n * c.h * c.w;
+    const uint32_t* am = at<uint32_t>(f, f.o.am[l]);
+    const bf16* yl = l == 2 ? at<bf16>(f, f.o.p3) : at<bf16>(f, f.o.p[l]);  // the pooled map
+    float* db = G + kOffB[l];
+    if (l == 0) {  // no input gradient: both of its sums come from the pooled gradient
+      k_dw1<<<dim3(static_cast<unsigned>(n), kDw1Parts), 256, 0, s>>>(x, at<bf16>(f, f.o.dp[0]), yl, am, G + kOffW[0], db);
+      f.launches++;
+      break;
+    }
     bf16* dyT = at<bf16>(f, f.o.dyT[l]);
-    bf16* dy = l > 0 ? at<bf16>(f, f.o.dy[l]) : nullptr;
+    bf16* dy = at<bf16>(f, f.o.dy[l]);
     {
       // the routed gradient and, fused, the bias gradient
       const dim3 ub(static_cast<unsigned>((m / 4 + 255) / 256), static_cast<unsigned>(c.cout / 16));
-      const uint32_t* am = at<uint32_t>(f, f.o.am[l]);
-      const bf16* yl = l == 2 ? at<bf16>(f, f.o.p3) : at<bf16>(f, f.o.p[l]);  // the pooled map
-      float* db = G + kOffB[l];
-      if (l == 0) {
-        k_unpool<16, true><<<ub, 256, 0, s>>>(at<bf16>(f, f.o.dp[l]), am, yl, n, c.h, c.w, dyT, dy, db);
-      } else if (l == 1) {
+      if (l == 1) {
         k_unpool<32, true><<<ub, 256, 0, s>>>(at<bf16>(f, f.o.dp[l]), am, yl, n, c.h, c.w, dyT, dy, db);
       } else {
         k_unpool<64, false><<<ub, 256, 0, s>>>(at<float>(f, f.o.dp3), am, yl, n, c.h, c.w, dyT, dy, db);
@@ -1827,12 +1854,6 @@ int backward(Sifter& f, const float* x, const float* y, int n, cudaStream_t s) {
     }
     f.launches++;
     // weight gradient
-    if (l == 0) {
-      static_assert(kW == 256 && kH + 2 <= 256, "k_dw1 geometry");
-      k_dw1<<<dim3(static_cast<unsigned>(n), 4), 256, 0, s>>>(x, n, dyT, G + kOffW[0]);
-      f.launches++;
-      break;
-    }
     bf16* S = at<bf16>(f, f.o.s3[l]);
     {
       const unsigned sg = static_cast<unsigned>(std::min<long long>((m / 8 * (c.cin / 2) + 255) / 256, 152LL * 8));
