@@ -485,8 +485,9 @@ def zfloat_rate(g, args, dev, dchunks, freqs, dms):
         bpu = W.nchan / W.ndm * es + 4.0  # payload ring read once per DM tile set + FP32 plane written
         peaks, src = _peaks()
         ach = bpu * W.chunk * W.ndm / (tms / 1e3) / 1e9
-        # its real bound: one shared-memory read of es bytes per (DM, sample, channel) against
-        # SMs x 128 bytes per clock at the maximum SM clock
+        # the reads of a tree that adds every channel for every DM, es bytes per (DM, sample, channel),
+        # against SMs x 128 bytes per clock at the maximum SM clock (summing shared leaf patterns
+        # once reads less: the fraction compares forms, it is not a share of the pipe)
         props = torch.cuda.get_device_properties(dev)
         smem_peak = props.multi_processor_count * 128 * float(peaks.get("sm_max_mhz") or 2070.0) * 1e6 / 1e9
         smem_ach = W.nchan * es * W.chunk * W.ndm / (tms / 1e3) / 1e9
@@ -494,9 +495,9 @@ def zfloat_rate(g, args, dev, dchunks, freqs, dms):
                      "tree_gdm_samples_per_s": round(W.chunk * W.ndm / (tms / 1e3) / 1e9, 2),
                      "roofline": {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                                   "frac": ach / peaks["hbm_gbs"], "peak_source": src,
-                                  "algorithmic_bytes_per_dm_sample": bpu, "kernel": "k_tree_z"},
+                                  "algorithmic_bytes_per_dm_sample": bpu, "kernel": "k_tree_zs"},
                      "roofline_smem": {"bound": "smem", "achieved": smem_ach, "peak": smem_peak, "unit": "GB/s",
-                                       "frac": smem_ach / smem_peak, "kernel": "k_tree_z",
+                                       "frac": smem_ach / smem_peak, "kernel": "k_tree_zs",
                                        "peak_source": f"derived: {props.multi_processor_count} SMs x 128 B/clock x "
                                                       "max SM clock",
                                        "algorithmic_bytes_per_dm_sample": W.nchan * es}}
