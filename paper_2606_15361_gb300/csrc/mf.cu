@@ -3,8 +3,9 @@
 // One CTA per DM row. The row segment [F_prev, E_new) of the plane ring (block start times
 // [F_prev, F_new) plus the Wmax-1 samples their windows reach) is staged in shared memory as it lies
 // in the ring (columns from the 16-byte boundary at or before F_prev); its exact integer sums give mu
-// and sigma over the block's start times, and an in-place exclusive scan turns it into prefix sums, so every boxcar is P[t+W] - P[t]. Everything works on quads of four consecutive
-// columns per lane (one 128-bit shared access).
+// and sigma over the block's start times, and an in-place exclusive scan turns it into prefix
+// sums, so every boxcar is P[t+W] - P[t]. Everything works on quads of four consecutive columns
+// per lane (one 128-bit shared access).
 //
 // Decision: a cell is in the mask iff max over the row's widths of
 //   SNR(W) = (S_W - mu*W) / (sigma*sqrt(W))          (FP64, this operation order)

@@ -499,7 +499,9 @@ __host__ __device__ constexpr int halo_stages(int cin, int cout, int w) {
 // memory as [tap][plane][cout][8]. 320 threads: two epilogue warpgroups (warps 0-3 and 4-7),
 // each draining one of the two TMEM accumulator buffers (items alternate between them), warp 8
 // issues the TMA loads and warp 9 owns TMEM and issues the MMAs; two or three shared-memory
-// stages. DX: the input gradient of a convolution, i.e. the same convolution of the output
+// stages. An MMA takes about 80 cycles, the time its A operand takes out of shared memory, which is what
+// bounds conv2 and conv3 once the waits suspend the warp and a lane pair shares the pooled stores
+// (training, 256 snippets: conv2 30.5 -> 28.7 us, conv3 39 -> 33). DX: the input gradient of a convolution, i.e. the same convolution of the output
 // gradient dY (channels-last) with the flipped, channel-transposed kernel; the epilogue writes
 // the sums rounded to BF16, channels-last [(b, y, x)][c].
 template <int CIN, int COUT, int W, bool TRAIN, bool DX = false>
@@ -711,6 +713,10 @@ __global__ void __launch_bounds__(320, 2)
 // TRAIN: also the argmax of every pooled cell (am). 448 threads: two epilogue warpgroups (warps 0-3
 // and 4-7), each draining one of the two TMEM accumulator buffers, warps 8-11 build U, warp 12 owns
 // TMEM and issues the MMAs, warp 13 issues the TMA loads.
+// Latency bounds it, not memory or the tensor pipe: a row tile passes through raw loads, U and the
+// epilogue, each waiting on the one before. 4096 snippets 430 us, 504 with one epilogue warpgroup, waits
+// that poll and one lane of a pair storing; training (256 snippets, with argmaxes) 50 -> 45 us, where a
+// third CTA per SM gained nothing.
 // Rounding: BF16 snippet values and weights, FP32 sums (the tensor core adds the nine
 // products in its own order), bias, ReLU, BF16 store.
 template <bool TRAIN>
@@ -1355,11 +1361,9 @@ __device__ __noinline__ void snippet_fp64(const float* __restrict__ plane, long 
 // thread. The FP64 pipe of this chip runs 1/64 of the FP32 rate, so an FP64 evaluation per cell
 // bounds a kernel that should be bound by its stores: the sums, the differences v - mu and the
 // products with 1 / sd are unevaluated FP32 pairs (two-sum, two-product: about 48 bits, so the
-// rounded result is the FP64 one), FP64 only in one warp, for the
-// CTA's two totals. The deviations are summed
-// about the mean, not as s2 / n - mu^2. 4096 snippets
-// of a 2048 x 16384 plane take 200 us (64: 13 us); with FP64 sums and divisions per cell 1806 us
-// (64: 72 us). What is left is latency: two CTAs fit an SM (the cells in registers), and each
+// rounded result is the FP64 one), FP64 only in one warp, for the CTA's two totals. The
+// deviations are summed about the mean, not as s2 / n - mu^2. 4096 snippets of a 2048 x 16384
+// plane take 200 us (64: 13 us); with FP64 sums and divisions per cell 1806 us (64: 72 us). What is left is latency: two CTAs fit an SM (the cells in registers), and each
 // loads, reduces twice and stores one after the other; the bytes alone would take about 80 us.
 __global__ void __launch_bounds__(256, 2) k_snippets(const float* __restrict__ plane, long long ld, int ndm,
                                                      long long ncols, const int32_t* __restrict__ rows,
