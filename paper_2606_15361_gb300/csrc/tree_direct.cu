@@ -19,12 +19,13 @@
 //
 // GPU mapping:
 //  * lanes are 32 consecutive trial DMs; a warp owns KW consecutive 32-sample words of the
-//    CTA's time tile (warp w: words w*KW ..), so per channel a lane reads one table entry (its byte
-//    offset among the round's windows and the bit shift: one add gives the address; a 16-bit word
-//    offset per channel took three instructions) and then KW+1 consecutive window words (a sliding
-//    funnel-shift window). The 32 DMs of a
-//    tile read one channel at offsets that differ by less than 32 words, so the reads hit
-//    distinct banks (or broadcast) without conflicts.
+//    CTA's time tile (warp w: words w*KW ..), so per channel a lane reads one table entry and then
+//    KW+1 consecutive window words (a sliding funnel-shift window). An entry is the window's byte
+//    offset among the round's windows and the bit shift: one add gives the address, where a 16-bit
+//    word offset per channel took three instructions (25 -> 22 a channel and warp; tree 307 -> 295 us
+//    float, 345 -> 333 graded for 1024 channels x 2048 DMs x 16384 samples: the ALU pipe, 76% busy,
+//    bounds it). The 32 DMs of a tile read one channel at offsets that differ by less than 32 words,
+//    so the reads hit distinct banks (or broadcast) without conflicts.
 //  * channels are staged 64 or 128 at a time (a round): every warp issues TMA bulk copies
 //    (cp.async.bulk) of its share of the round's channel windows from the L2-resident bit
 //    ring, and warp 0 the round's offset table, onto a double-buffered mbarrier pipeline, so
