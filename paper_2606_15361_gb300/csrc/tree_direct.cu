@@ -23,7 +23,7 @@
 //    KW+1 consecutive window words (a sliding funnel-shift window). An entry is the window's byte
 //    offset among the round's windows and the bit shift: one add gives the address, where a 16-bit
 //    word offset per channel took three instructions (25 -> 22 a channel and warp; tree 307 -> 295 us
-//    float, 345 -> 333 graded for 1024 channels x 2048 DMs x 16384 samples: the ALU pipe, 76% busy,
+//    float, 345 -> 333 graded for 1024 channels x 2048 DMs x 16384 samples: the ALU pipe, 78% busy,
 //    bounds it). The 32 DMs of a tile read one channel at offsets that differ by less than 32 words,
 //    so the reads hit distinct banks (or broadcast) without conflicts.
 //  * channels are staged 64 or 128 at a time (a round): every warp issues TMA bulk copies
