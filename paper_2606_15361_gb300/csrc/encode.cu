@@ -291,8 +291,21 @@ struct EncMulti {
   EncBeam beam[kMaxEncBeams];
 };
 
-// shared memory of a CTA: the samples and the packed words
+// dynamic shared memory of a CTA: the samples and the packed words
 __host__ __device__ constexpr int enc_smem(int wpc) { return wpc * 32 * 32 + 32 * (wpc | 1) * 4; }
+
+// static shared memory of a CTA of NT threads
+template <int NT>
+struct EncShared {
+  uint32_t red[NT / 32][4][32];
+  // every CTA's totals: sum and sum of squares; count below, count above, sum and sum of squares of both
+  uint32_t tot1[kEncCluster][2][32], tot2[kEncCluster][4][32];
+  int clip[2][32], lev[32];
+};
+
+// Longest chunk of the one-launch encoder: what a CTA may have in shared memory less its static part
+// (217,728 bytes: 189 ring words a CTA, 1512 a cluster, 48,384 samples from a word's start).
+constexpr int kEncMaxSmem = 227 * 1024 - static_cast<int>(sizeof(EncShared<512>));
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -330,10 +343,12 @@ __device__ __forceinline__ void cluster_put(uint32_t addr, uint32_t v, int S) {
 template <int kEncThreads>
 __device__ __forceinline__ void encode_cta(const EncBeam& e, const int cb, unsigned char* sm) {
   constexpr int NW = kEncThreads / 32;
-  __shared__ uint32_t red[NW][4][32];
-  // every CTA's totals: sum and sum of squares; count below, count above, sum and sum of squares of both
-  __shared__ uint32_t tot1[kEncCluster][2][32], tot2[kEncCluster][4][32];
-  __shared__ int clip[2][32], lev[32];
+  __shared__ EncShared<kEncThreads> sh;
+  auto &red = sh.red;
+  auto &tot1 = sh.tot1;
+  auto &tot2 = sh.tot2;
+  auto &clip = sh.clip;
+  auto &lev = sh.lev;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int rank = static_cast<int>(cluster_rank()), S = static_cast<int>(cluster_size());
   unsigned char* tile = sm;                                // [wpc * 32][32]
@@ -595,7 +610,7 @@ bool enc_beam(const Plan& p, const uint8_t* chunk, int nsamp, int S, EncBeam& e)
   const uintptr_t at = reinterpret_cast<uintptr_t>(chunk) | static_cast<uintptr_t>(p.nchan);
   e.vec = (at & 15u) == 0 ? 16 : ((at & 3u) == 0 ? 4 : 1);
   e.counters = p.dp.counters;
-  return enc_smem(e.wpc) <= 220 * 1024 && e.nwords <= e.R;
+  return enc_smem(e.wpc) <= kEncMaxSmem && e.nwords <= e.R;
 }
 
 template <typename A>
