@@ -282,8 +282,6 @@ struct EncBeam {
 
 constexpr int kMaxEncBeams = 64;
 constexpr int kEncCluster = 8;  // most CTAs of a cluster
-// A CTA of 256 threads where four fit an SM's shared memory, of 512 where fewer do.
-constexpr int kEncSmall = 54 * 1024;
 
 struct EncMulti {
   int nbeams;
@@ -306,6 +304,15 @@ struct EncShared {
 // Longest chunk of the one-launch encoder: what a CTA may have in shared memory less its static part
 // (217,728 bytes: 189 ring words a CTA, 1512 a cluster, 48,384 samples from a word's start).
 constexpr int kEncMaxSmem = 227 * 1024 - static_cast<int>(sizeof(EncShared<512>));
+// The most dynamic shared memory with which `ctas` CTAs of NT threads fit an SM (228 KB, of which a CTA
+// takes its dynamic and static parts and 1 KB).
+template <int NT>
+constexpr int enc_fit(int ctas) { return 228 * 1024 / ctas - 1024 - static_cast<int>(sizeof(EncShared<NT>)); }
+// A CTA of 256 threads where three fit an SM, of 512 where fewer do: 4096 channels take 57 us with
+// three of 256 threads and 64 with two of 512 (12,500 samples; 62 and 71 at 14,300), and 63 against 54
+// where even 512 threads fit three times (11,000 samples).
+constexpr int kEncSmall = enc_fit<256>(3);  // 66,176 bytes: 57 words a CTA
+constexpr int kEncTwo = enc_fit<512>(2);    // 100,992 bytes: 87 words
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -683,14 +690,23 @@ cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cuda
   return cudaGetLastError();
 }
 
-// Encoders of several plans in one launch per shared-memory class (54 KB a CTA: four fit an SM;
-// 110 KB: two; more: one), so a long-chunk beam does not lower every other beam's occupancy; more
-// launches only past kMaxEncBeams beams of a class. Plans that k_encode does not take run their own
-// launch_encode.
+// Encoders of several plans in one launch per shared-memory class (three CTAs fit an SM, two, one), so
+// a long-chunk beam does not lower every other beam's occupancy: eight beams of 1024 channels, one with
+// 24,000 samples and seven with 22,000, take 498 us a step in one launch and 417 in two. Beams of which
+// all CTAs fit the GPU one per SM need no such care, and save the launch. More launches only past
+// kMaxEncBeams beams of a class. Plans that k_encode does not take run their own launch_encode.
 cudaError_t launch_encode_batch(const Plan* const* plans, const uint8_t* const* chunks, const int32_t* nsamp, int n,
                                 cudaStream_t s) {
   constexpr int S = kEncCluster;
-  auto cls = [](int smem) { return smem <= kEncSmall ? 0 : (smem <= 110 * 1024 ? 1 : 2); };
+  int dev = 0, nsm = 0, wide = 0;  // wide: CTAs that fit fewer than three times
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) return err;
+  for (int i = 0; i < n; ++i) {
+    EncBeam b{};
+    if (enc_beam(*plans[i], chunks[i], nsamp[i], S, b) && enc_smem(b.wpc) > kEncSmall) wide += (plans[i]->nchan + 31) / 32 * S;
+  }
+  auto cls = [&](int smem) { return smem <= kEncSmall ? 0 : (smem <= kEncTwo || wide <= nsm ? 1 : 2); };
   EncMulti m{};
   int clusters = 0, smem = 0;
   const Plan* owner = nullptr;

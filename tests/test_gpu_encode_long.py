@@ -56,3 +56,32 @@ def test_spikes_of_the_longest_chunks(n, before, nchan, batch):
             assert (got[1:32] == got[0]).all()
         done += ne
     assert plan.candidates()[1] == 0
+
+
+@pytest.mark.parametrize("lengths", [
+    (14592, 14593, 22272, 22273),                  # few CTAs: the beams of more than 14,592 samples in one launch
+    (14592, 14593, 22272, 22273, 22273, 20000),    # more than the GPU takes one per SM: a launch per class
+])
+def test_batch_of_every_class(lengths):
+    """Beams on both sides of the lines between three, two and one CTA per SM."""
+    nchan, rng = 160, np.random.default_rng(len(lengths))
+    freqs = synth.channel_freqs(nchan)
+    plans, spikes, devs, delays = [], [], [], []
+    for n in lengths:
+        dms = DMS * (n / 47000.0)  # a sweep of about a chunk
+        delays.append(odelays.delay_table(freqs, synth.NC_DT, dms))
+        plans.append(g.Plan(freqs, synth.NC_DT, dms, 4, g.MODE_FLOAT,
+                            g.options(g.MODE_FLOAT, enc_theta=THETA, det_theta=1e6, max_chunk=n)))
+        x = [np.clip(np.rint(rng.normal(128, 16, (n, nchan))), 0, 255).astype(np.uint8) for _ in range(2)]
+        spikes.append(np.concatenate([oenc.encode_chunk(c, THETA)[0].astype(np.int64) for c in x], axis=1))
+        devs.append([torch.from_numpy(c).cuda() for c in x])
+    done = [p.nemit_next(n) for p, n in zip(plans, lengths)]
+    g.Batch(plans).execute([d[0] for d in devs])
+    for p, n, s, d, t, delay in zip(plans, lengths, spikes, devs, done, delays):
+        ne = p.nemit_next(n)
+        out = torch.full((len(DMS), max(ne, 1)), -1.0, dtype=torch.float32, device="cuda")
+        assert p.execute(d[1], out) == ne
+        got = np.rint(out[:, :ne].cpu().numpy().astype(np.float64) * np.sqrt(nchan)).astype(np.int64)
+        for r in (0, 32):
+            assert np.array_equal(got[r], sum(s[c, t + delay[r, c]:t + delay[r, c] + ne] for c in range(nchan)))
+        assert p.candidates()[1] == 0
