@@ -468,31 +468,50 @@ __global__ void k_emit(const int32_t* row_runs, int ndm, int run_cap, const int3
              blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// Rank every block candidate by (t, dm_index) (keys are distinct: one peak pixel per island)
-// and place it after the candidates already held.
+// Rank every block candidate by (t, dm_index) (keys are distinct: one peak pixel per island) and place it
+// after the candidates already held. Called by whole CTAs of 256 threads: a CTA takes the candidates
+// i0, i0 + stride, ... and the 255 after each, and brings the keys through shared memory (`keys`,
+// kRankTile words), from where four are compared per load. Read from the list itself, field by field, a
+// block of 1400 candidates took one CTA 0.5 ms, and one of 34,000 a small grid 3 ms.
+constexpr int kRankTile = 2048;
 __device__ __forceinline__ void rank_items(const snd_candidate_t* bcand, snd_candidate_t* cand, uint32_t* counters,
-                                           int cand_cap, int i0, int stride) {
+                                           int cand_cap, int ndm, long long f_prev, uint32_t* keys, int i0,
+                                           int stride) {
   const int n = min(static_cast<int>(counters[kCntBlockCands]), cand_cap);
   const int base = static_cast<int>(counters[kCntCands]);
-  for (int i = i0; i < n; i += stride) {
-    const snd_candidate_t ci = bcand[i];
+  // the position in the block, sample by sample: below ndm * nb, which fits 32 bits
+  auto key_of = [&](const snd_candidate_t& c) {
+    return static_cast<uint32_t>(c.t - f_prev) * static_cast<uint32_t>(ndm) + static_cast<uint32_t>(c.dm_index);
+  };
+  for (int ib = i0; ib < n; ib += stride) {
+    const int i = ib + static_cast<int>(threadIdx.x);
+    const uint32_t key = i < n ? key_of(bcand[i]) : 0u;
     int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const snd_candidate_t cj = bcand[j];
-      rank += (cj.t < ci.t) || (cj.t == ci.t && cj.dm_index < ci.dm_index);
+    for (int j0 = 0; j0 < n; j0 += kRankTile) {
+      const int m = (min(kRankTile, n - j0) + 3) & ~3;
+      __syncthreads();
+      for (int j = threadIdx.x; j < m; j += 256) keys[j] = j0 + j < n ? key_of(bcand[j0 + j]) : 0xFFFFFFFFu;
+      __syncthreads();
+#pragma unroll 4
+      for (int j = 0; j < m; j += 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(keys + j);
+        rank += (q.x < key) + (q.y < key) + (q.z < key) + (q.w < key);
+      }
     }
+    if (i >= n) continue;
     const int pos = base + rank;
     if (pos < cand_cap) {
-      cand[pos] = ci;
+      cand[pos] = bcand[i];
     } else {
       atomicOr(&counters[kCntStatus], kStatusCandOverflow);
     }
   }
 }
 
-__global__ void k_rank_append(const snd_candidate_t* bcand, snd_candidate_t* cand, uint32_t* counters,
-                              int cand_cap) {
-  rank_items(bcand, cand, counters, cand_cap, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+__global__ void __launch_bounds__(256) k_rank_append(const snd_candidate_t* bcand, snd_candidate_t* cand,
+                                                     uint32_t* counters, int cand_cap, int ndm, long long f_prev) {
+  __shared__ __align__(16) uint32_t keys[kRankTile];
+  rank_items(bcand, cand, counters, cand_cap, ndm, f_prev, keys, blockIdx.x * 256, gridDim.x * 256);
 }
 
 __device__ __forceinline__ void bump(uint32_t* counters, int cand_cap) {
@@ -602,6 +621,7 @@ __device__ __forceinline__ bool grid_last(const CandMulti& m) {
 // A block of at most this many runs (the usual block has a few hundred) has its islands joined by one
 // CTA in shared memory: a root walk there takes tens of cycles a step, in global memory hundreds.
 constexpr int kSmallRuns = 2048;
+static_assert(kRankTile <= 4 * kSmallRuns, "the ranking's keys take the join's place in shared memory");
 
 __device__ __forceinline__ void join_small(const CandBeam& e, int n, uint32_t* csm) {
   int* par = reinterpret_cast<int*>(csm);
@@ -632,7 +652,7 @@ __device__ __forceinline__ void join_small(const CandBeam& e, int n, uint32_t* c
 // 38 -> 29, 128 x 16384 65 -> 50, 2048 x 16384 binary 56 -> 48, graded 113 -> 66, float 81 -> 57; eight
 // beams (one launch) 517 -> 315.
 __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ CandMulti m) {
-  extern __shared__ uint32_t csm[];
+  extern __shared__ __align__(16) uint32_t csm[];
   const int nblk = gridDim.x, bid = blockIdx.x, tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int gtid = bid * 256 + tid, gthreads = nblk * 256;
@@ -729,7 +749,7 @@ __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ Cand
     emit_items(e0.row_runs, e0.ndm, e0.run_cap, e0.parent, e0.npix, e0.peak, e0.pwidth, e0.nb, e0.n_min, e0.f_prev,
                e0.dm_f32, e0.bcand, e0.cand_cap, e0.counters, tid, 256);
     __syncthreads();
-    rank_items(e0.bcand, e0.cand, e0.counters, e0.cand_cap, tid, 256);
+    rank_items(e0.bcand, e0.cand, e0.counters, e0.cand_cap, e0.ndm, e0.f_prev, csm, 0, 256);
     __syncthreads();
     if (tid == 0) bump(e0.counters, e0.cand_cap);
     return;
@@ -743,7 +763,7 @@ __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ Cand
   if (!grid_barrier(m)) return;
   for (int b = 0; b < m.nbeams; ++b) {
     const CandBeam& e = m.beam[b];
-    rank_items(e.bcand, e.cand, e.counters, e.cand_cap, gtid, gthreads);
+    rank_items(e.bcand, e.cand, e.counters, e.cand_cap, e.ndm, e.f_prev, csm, bid * 256, gthreads);
   }
   if (!grid_barrier(m)) return;
   for (int b = gtid; b < m.nbeams; b += gthreads) bump(m.beam[b].counters, m.beam[b].cand_cap);
@@ -803,7 +823,7 @@ cudaError_t launch_candidates(const Plan& p, int64_t f_prev, int nb, cudaStream_
                                      dp.run_start, dp.run_end, dp.parent, dp.peak, dp.pwidth, 1);
   k_emit<<<kGridStride, 256, 0, s>>>(dp.row_runs, p.ndm, p.run_cap, dp.parent, dp.npix, dp.peak, dp.pwidth, nb,
                                      p.n_min, f_prev, dp.dm_f32, dp.bcand, p.cand_cap, dp.counters);
-  k_rank_append<<<kGridStride, 256, 0, s>>>(dp.bcand, dp.cand, dp.counters, p.cand_cap);
+  k_rank_append<<<kGridStride, 256, 0, s>>>(dp.bcand, dp.cand, dp.counters, p.cand_cap, p.ndm, f_prev);
   k_bump<<<1, 1, 0, s>>>(dp.counters, p.cand_cap);
   p.launches += 11;
   return cudaGetLastError();
