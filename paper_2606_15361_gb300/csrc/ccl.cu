@@ -621,6 +621,10 @@ __device__ __forceinline__ bool grid_last(const CandMulti& m) {
 // A block of at most this many runs (the usual block has a few hundred) has its islands joined by one
 // CTA in shared memory: a root walk there takes tens of cycles a step, in global memory hundreds.
 constexpr int kSmallRuns = 2048;
+// A block of at most this many has its candidates emitted and ranked by one CTA, which saves two
+// barriers (stage us, one CTA / the whole grid: 57 candidates 32 / 38, 340 45 / 47, 541 58 / 53, 867 73 / 54,
+// 1446 120 / 68).
+constexpr int kFewRuns = 512;
 static_assert(kRankTile <= 4 * kSmallRuns, "the ranking's keys take the join's place in shared memory");
 
 __device__ __forceinline__ void join_small(const CandBeam& e, int n, uint32_t* csm) {
@@ -744,7 +748,7 @@ __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ Cand
     if (pass == 0 && !grid_barrier(m)) return;
   }
   // 6. the block's candidates, ranked and appended
-  if (one && !large) {
+  if (one && runs_of(e0) <= kFewRuns) {
     if (!grid_last(m)) return;
     emit_items(e0.row_runs, e0.ndm, e0.run_cap, e0.parent, e0.npix, e0.peak, e0.pwidth, e0.nb, e0.n_min, e0.f_prev,
                e0.dm_f32, e0.bcand, e0.cand_cap, e0.counters, tid, 256);

@@ -1,5 +1,5 @@
 """Blocks of an exact number of runs and islands around the lines where the candidate stage changes its
-form: 2048 runs (islands joined, and candidates ranked, by one CTA or by the whole grid), 2048 keys a
+form: 2048 runs (islands joined) and 512 runs (candidates ranked by one CTA or the whole grid), 2048 keys a
 shared-memory tile of the ranking, 256 candidates a CTA. Every channel fires at isolated samples of an
 otherwise constant chunk, so a row has one run per sample, and equal trial DMs join their rows' runs.
 Two blocks a plan (the second list is appended), alone and in a batch; lists equal the C++ oracle's."""
@@ -37,8 +37,9 @@ def _tuples(cands):
 
 
 @pytest.mark.parametrize("reference", [False, True], ids=["cooperative", "staged"])
-@pytest.mark.parametrize("ndm,islands", [(1, 1), (1, 255), (1, 256), (1, 257), (1, 2047), (1, 2048), (1, 2049),
-                                         (2, 1024), (2, 1025), (3, 682), (3, 683), (5, 2060)])
+@pytest.mark.parametrize("ndm,islands", [(1, 1), (1, 255), (1, 256), (1, 257), (1, 511), (1, 512), (1, 513),
+                                         (1, 2047), (1, 2048), (1, 2049), (2, 1024), (2, 1025), (3, 682), (3, 683),
+                                         (5, 2060)])
 def test_blocks_around_the_lines(ndm, islands, reference):
     chunks = [_chunk(islands, 300), _chunk(max(1, islands - 3), 57)]
     cfg = ostream.defaults(ostream.FLOAT, branching=2, det_theta=3.5, n_min=1, closing=1, sigma_min=0.0)
