@@ -648,7 +648,11 @@ cudaError_t launch_encode(const Plan& p, const uint8_t* d_chunk, int nsamp, cuda
     int S = kEncCluster;
     while (S > 1 && nwords < 8 * S) S /= 2;
     EncBeam b{};
-    if (enc_beam(p, d_chunk, nsamp, S, b)) {
+    // A few channels read byte by byte are one or two clusters, whose CTAs' loads take longer than the three
+    // launches that spread a long chunk over the GPU (stage us, one launch / three: 7 channels x 26,000 samples
+    // 28 / 26, 48,000 39 / 26; 33 x 26,000 29 / 31, 48,000 37 / 31; 66 x 48,000 37 / 35).
+    const bool long_bytes = p.nchan <= 64 && nwords > 104 * kEncCluster;
+    if (enc_beam(p, d_chunk, nsamp, S, b) && !(b.vec == 1 && long_bytes)) {
       p.launches += 1;
       const int smem = enc_smem(b.wpc), clusters = (p.nchan + 31) / 32;
       return smem <= kEncSmall ? run_encode(k_encode<256>, 256, b, clusters, S, smem, s)
