@@ -301,8 +301,8 @@ extern "C" int snd_multirate_plan(const double* freqs_mhz, int32_t nchan, double
   m->off_parent = take(sizeof(int32_t) * cap_total);
   m->off_best = take(sizeof(uint32_t) * cap_total);
   m->off_tie = take(sizeof(unsigned long long) * cap_total);
+  m->off_cnt = take(snd::kReadHead);  // the merged list follows it (HostRead)
   m->off_out = take(sizeof(snd_candidate_t) * cap_total);
-  m->off_cnt = take(sizeof(uint32_t) * 4);
   m->off_dm = take(sizeof(double) * ndm);
   m->off_native = take(static_cast<size_t>(o.max_chunk) * nchan);
   m->ws_bytes = off;
@@ -481,17 +481,15 @@ extern "C" int snd_multirate_candidates(snd_multirate_t h, snd_candidate_t* host
   k_best<<<64, 256, 0, s>>>(all, cnt, m.cap, parent, best, tie, 1);
   k_emit_sorted<<<64, 256, 0, s>>>(all, cnt, m.cap, parent, best, tie, outd, cnt + 1);
   if (cudaGetLastError() != cudaSuccess) return fail(m, SND_ERR_CUDA);
-  if (!m.read.ready()) return fail(m, SND_ERR_NOMEM);
-  const uint32_t* hc = m.read.counters;
+  const uint32_t* hc = m.read.counters();
   const int head = static_cast<int>(std::min<int64_t>(std::min<int64_t>(cap, m.cap), snd::kReadCands));
-  if (cudaMemcpyAsync(m.read.counters, cnt, sizeof(uint32_t) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      (head > 0 && cudaMemcpyAsync(m.read.cand, outd, sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
-                       cudaSuccess) ||
+  if (cudaMemcpyAsync(m.read.buf, cnt, snd::kReadHead + sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return fail(m, SND_ERR_CUDA);
   const int n = static_cast<int>(hc[1]);
   const int take = std::min(n, cap);
-  if (take > 0) std::memcpy(host_out, m.read.cand, sizeof(snd_candidate_t) * std::min(take, head));
+  if (take > 0) std::memcpy(host_out, m.read.cand(), sizeof(snd_candidate_t) * std::min(take, head));
   if (snd::read_tail(outd, take, host_out, s) != cudaSuccess) return fail(m, SND_ERR_CUDA);
   *n_out = take;
   const uint32_t st = hc[2] | hc[3];

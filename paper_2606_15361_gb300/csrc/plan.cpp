@@ -310,7 +310,8 @@ int build_plan(Plan& p) {
   p.off.mask2 = take(sizeof(uint32_t) * static_cast<size_t>(ndm) * p.mw);
   p.off.mask3 = take(sizeof(uint32_t) * static_cast<size_t>(ndm) * p.mw);
   p.off.cells = take(sizeof(MfCell) * static_cast<size_t>(p.cell_cap));
-  p.off.counters = take(sizeof(uint32_t) * kCntSlots);
+  p.off.counters = take(kReadHead);  // the candidate list follows them (HostRead)
+  p.off.cand = take(sizeof(snd_candidate_t) * static_cast<size_t>(p.cand_cap));
   p.off.row_runs = take(sizeof(int32_t) * (static_cast<size_t>(ndm) + 1));
   p.off.run_start = take(sizeof(int32_t) * static_cast<size_t>(p.run_cap));
   p.off.run_end = take(sizeof(int32_t) * static_cast<size_t>(p.run_cap));
@@ -320,7 +321,6 @@ int build_plan(Plan& p) {
   p.off.peak = take(sizeof(unsigned long long) * static_cast<size_t>(p.run_cap));
   p.off.pwidth = take(sizeof(int32_t) * static_cast<size_t>(p.run_cap));
   p.off.bcand = take(sizeof(snd_candidate_t) * static_cast<size_t>(p.cand_cap));
-  p.off.cand = take(sizeof(snd_candidate_t) * static_cast<size_t>(p.cand_cap));
   p.off.staging = take(static_cast<size_t>(p.max_chunk) * nchan);
   p.off.staging2 = take(static_cast<size_t>(p.max_chunk) * nchan);
   p.off.width_mask = take(sizeof(uint16_t) * ndm);

@@ -8,7 +8,6 @@
 
 #include <algorithm>
 #include <cstring>
-#include <new>
 #include <vector>
 
 #include "snd_internal.h"
@@ -33,29 +32,6 @@ void chunk_commit(Plan& p, const ChunkPos& c, int32_t nsamp, cudaStream_t s) {
   p.F = (p.mode == SND_MODE_ZFLOAT) ? p.F : c.f_new;
   p.last_stream = s;
   p.pending_host = -1;
-}
-
-bool HostRead::ready() {
-  if (counters) return true;
-  constexpr size_t head = 64, bytes = head + sizeof(snd_candidate_t) * kReadCands;
-  static_assert(sizeof(uint32_t) * kCntSlots <= head, "counters before the candidates");
-  void* m = nullptr;
-  if (cudaHostAlloc(&m, bytes, cudaHostAllocPortable) != cudaSuccess) {
-    cudaGetLastError();
-    try {
-      pageable.resize(bytes + alignof(snd_candidate_t));
-    } catch (const std::bad_alloc&) {
-      return false;
-    }
-    m = pageable.data();
-  }
-  counters = static_cast<uint32_t*>(m);
-  cand = reinterpret_cast<snd_candidate_t*>(static_cast<unsigned char*>(m) + head);
-  return true;
-}
-
-HostRead::~HostRead() {
-  if (counters && pageable.empty()) cudaFreeHost(counters);
 }
 
 cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s) {
@@ -94,6 +70,13 @@ cudaError_t mark(Plan& p, cudaStream_t s, size_t* slot) {
   }
   *slot = p.ev_used++;
   return cudaEventRecord(p.ev_pool[*slot], s);
+}
+
+// The counters go to their second copy, and the list's count and status word start afresh.
+__global__ void k_take_counters(uint32_t* counters) {
+  const int i = threadIdx.x;
+  counters[snd::kCntTaken + i] = counters[i];
+  if (i == snd::kCntCands || i == snd::kCntStatus) counters[i] = 0;
 }
 
 // Run one stage inside an NVTX range named for it (host-side enqueue time in a timeline
@@ -352,22 +335,21 @@ extern "C" int snd_candidates(snd_plan_t plan, snd_candidate_t* host_out, int32_
   Plan& p = *reinterpret_cast<Plan*>(plan);
   if (!p.bound) return SND_ERR_STATE;
   if (p.sticky) return p.sticky;
-  // the counters, the head of the list and the reset of its count and status word (adjacent) in the
-  // stream's order, one wait for all three
-  if (!p.read.ready()) return fail(p, SND_ERR_NOMEM);
+  // the counters are taken and the list's count and status word reset before the copy is enqueued, so one
+  // wait covers all three
   cudaStream_t s = p.last_stream;
-  const uint32_t* cnt = p.read.counters;
+  const uint32_t* cnt = p.read.counters() + snd::kCntTaken;
   const int head = std::min(std::min(cap, p.cand_cap), snd::kReadCands);
-  if (cudaMemcpyAsync(p.read.counters, p.dp.counters, sizeof(uint32_t) * snd::kCntSlots, cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
-      (head > 0 && cudaMemcpyAsync(p.read.cand, p.dp.cand, sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
-                       cudaSuccess) ||
-      cudaMemsetAsync(p.dp.counters + snd::kCntCands, 0, sizeof(uint32_t) * 2, s) != cudaSuccess ||
+  k_take_counters<<<1, snd::kCntSlots, 0, s>>>(p.dp.counters);
+  p.launches += 1;
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(p.read.buf, p.dp.counters, snd::kReadHead + sizeof(snd_candidate_t) * head,
+                      cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return fail(p, SND_ERR_CUDA);
   const int n = static_cast<int>(cnt[snd::kCntCands]);
   const int take = n < cap ? n : cap;
-  if (take > 0) std::memcpy(host_out, p.read.cand, sizeof(snd_candidate_t) * std::min(take, head));
+  if (take > 0) std::memcpy(host_out, p.read.cand(), sizeof(snd_candidate_t) * std::min(take, head));
   if (snd::read_tail(p.dp.cand, take, host_out, s) != cudaSuccess) return fail(p, SND_ERR_CUDA);
   *n_out = take;
   p.pending_host = 0;

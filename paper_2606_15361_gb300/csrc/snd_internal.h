@@ -184,21 +184,22 @@ enum {
   kCntStatus = 4,
   kCntTreeQueue = 8,   // many-beam tree: next work item (the first plan of a batch launch)
   kCntGridBar = 12,    // many-beam candidates: grid barrier arrivals, generation (two slots)
-  kCntSlots = 16
+  kCntSlots = 16,
+  kCntTaken = 16       // .. kCntTaken + kCntSlots: the counters as the last read took them
 };
 
-// Where a plan's counters and the head of its candidate list are read back to: page-locked, so both
-// copies and the reset of the list wait on the GPU once. Allocated at the first read, freed with its
-// owner. Candidate lists past kReadCands take a second copy.
-constexpr int kReadCands = 512;
+// Where counters and the head of a candidate list, which follow each other on the device, are read back to
+// in one copy; candidates past kReadCands go to the caller's buffer in a second one. Pageable on purpose: a
+// page-locked buffer saves 3 to 9 us of an idle read (18 us against 21 to 27) and nothing that shows beside a
+// chunk, but freeing it waits for all work on the GPU: destroying a plan took as long as other streams'
+// kernels (10 ms beside 20 matrix products; 7 us now), its first read 175 us (45 now).
+constexpr int kReadCands = 512, kReadHead = 256;
 struct HostRead {
-  uint32_t* counters = nullptr;      // [kCntSlots]
-  snd_candidate_t* cand = nullptr;   // [kReadCands]
-  std::vector<unsigned char> pageable;  // in use when page-locked memory is not to be had
-  bool ready();
-  ~HostRead();
+  alignas(16) unsigned char buf[kReadHead + sizeof(snd_candidate_t) * kReadCands];
+  const uint32_t* counters() const { return reinterpret_cast<const uint32_t*>(buf); }
+  const snd_candidate_t* cand() const { return reinterpret_cast<const snd_candidate_t*>(buf + kReadHead); }
 };
-// Head of the list: the n candidates at `src` (device) from kReadCands on go to host_out directly.
+// The candidates [kReadCands, take) of the list at `src` (device) to host_out.
 cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s);
 
 struct Plan {
