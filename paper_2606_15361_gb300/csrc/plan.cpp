@@ -283,7 +283,8 @@ int build_plan(Plan& p) {
   int rc = (p.mode == SND_MODE_ZFLOAT) ? choose_ztree_geometry(p) : choose_tree_geometry(p);
   if (p.mode != SND_MODE_ZFLOAT) {
     choose_direct_geometry(p);
-    // channel counts in whole groups: the leaf-sharing kernel may not fit, the direct one does
+    // channel counts in whole groups, windows that are not the widest: the leaf-sharing kernel may not fit, the
+    // direct one does
     if (p.direct && p.dgeom.whole) rc = SND_OK;
   }
   if (rc) return rc;
@@ -641,6 +642,10 @@ void choose_direct_geometry(Plan& p) {
     g.sgroups = (nc % 128 == 0 && smem_for(2) <= 112 * 1024) ? 2 : 1;
   const int64_t smem = smem_for(g.sgroups);
   if (smem > 220 * 1024) return;
+  // the widest windows (more than 200 KB with a table of 16-bit entries) run here only where the leaf-sharing
+  // kernel would take the plan; it is three to four times slower (1024 channels, windows of 380 to 400 words, 78 us
+  // against 297)
+  g.whole = g.whole && smem - 64 * g.sgroups * 32 * 4 <= 200 * 1024;
   g.smem_bytes = static_cast<int>(smem);
   p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nc * 32, 0);
   for (int t = 0; t < g.ndm_tiles; ++t)

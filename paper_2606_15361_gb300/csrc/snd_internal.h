@@ -84,7 +84,8 @@ enum {
 struct DirectGeom {
   int inst = kDirNone;
   int nchan = 0;         // channels rounded up to a multiple of 64 (the rest are zero ring rows)
-  bool whole = true;     // every exact-level node (all modes: the channel count) is whole 64-channel groups
+  bool whole = true;     // the plan stands even where the leaf-sharing kernel does not fit: every exact-level node
+                         // (all modes: the channel count) is whole 64-channel groups, and the windows are not the widest
   int warps = 8;
   int kw = 4;
   int tile_words = 32;   // warps * kw
