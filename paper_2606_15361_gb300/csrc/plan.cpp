@@ -522,8 +522,8 @@ int choose_tree_geometry_w(Plan& p, int warps) {
 // output words; channels are staged 64 at a time. Per (DM tile, channel) the first staged ring
 // word is base4 = (min over the tile of delta >> 5) rounded down to a multiple of 4 (16-byte
 // aligned bulk copies), and per (tile, channel, DM) the entry (byte offset of window word
-// (delta >> 5) - base4 among the windows of the channel's round) << 5 | delta & 31 gives the DM's
-// window word and funnel shift.
+// (delta >> 5) - base4 among the windows of the channel's round, or in 16 bits that word itself) << 5 |
+// delta & 31 gives the DM's window word and funnel shift.
 void choose_direct_geometry(Plan& p) {
   snd::DirectGeom& g = p.dgeom;
   g = snd::DirectGeom{};
@@ -632,22 +632,28 @@ void choose_direct_geometry(Plan& p) {
     }
   if (omax > 2047) return;
   g.cspan = static_cast<int>(align_up(static_cast<size_t>(4 + omax + g.warps * span_kw), 4));
-  // stage 128 channels per round (half the barriers) when they fit two CTAs per SM
-  auto smem_for = [&](int sg) { return (2 * 64 * sg * (static_cast<int64_t>(g.cspan) + 32) + nc) * 4; };
+  // The table's entries have 32 bits, or 16 where two CTAs fit an SM only with those (1024 channels: windows of
+  // 188 to 200 words; tree us, 32 / 16 bits, 512 DMs x 45,000 samples, float 324 / 290, graded 353 / 311, binary
+  // 328 / 288). 128 channels are staged per round (half the barriers) where two CTAs fit with 32-bit entries;
+  // with 16-bit ones at windows of 80 words it gains nothing over 64 (float 229 / 223, binary 215 / 214).
+  auto smem_for = [&](int sg, int bytes) {
+    return 2 * 64 * sg * (static_cast<int64_t>(g.cspan) * 4 + 32 * bytes) + nc * 4;
+  };
+  constexpr int64_t kTwo = 228 * 1024 / 2 - 1024 - 128;  // dynamic shared memory with which two CTAs fit an SM
   if (p.tree_round == 64)
     g.sgroups = 1;
   else if (p.tree_round == 128)
     g.sgroups = nc % 128 == 0 ? 2 : 1;
   else
-    g.sgroups = (nc % 128 == 0 && smem_for(2) <= 112 * 1024) ? 2 : 1;
-  const int64_t smem = smem_for(g.sgroups);
+    g.sgroups = (nc % 128 == 0 && smem_for(2, 4) <= 112 * 1024) ? 2 : 1;
+  g.narrow = smem_for(g.sgroups, 4) > kTwo && smem_for(g.sgroups, 2) <= kTwo;
+  const int64_t smem = smem_for(g.sgroups, g.narrow ? 2 : 4);
   if (smem > 220 * 1024) return;
-  // the widest windows (more than 200 KB with a table of 16-bit entries) run here only where the leaf-sharing
-  // kernel would take the plan; it is three to four times slower (1024 channels, windows of 380 to 400 words, 78 us
-  // against 297)
-  g.whole = g.whole && smem - 64 * g.sgroups * 32 * 4 <= 200 * 1024;
+  // the widest windows run here only where the leaf-sharing kernel would take the plan (it is three to four times
+  // slower: 1024 channels, windows of 380 to 400 words, 78 us against 297)
+  g.whole = g.whole && smem_for(g.sgroups, 2) <= 200 * 1024;
   g.smem_bytes = static_cast<int>(smem);
-  p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nc * 32, 0);
+  p.dmeta.assign(static_cast<size_t>(g.ndm_tiles) * nc * 32 / (g.narrow ? 2 : 1), 0);
   for (int t = 0; t < g.ndm_tiles; ++t)
     for (int c = 0; c < nc; ++c) {
       const int32_t b4 = p.dbase[static_cast<size_t>(t) * nc + c];
@@ -655,8 +661,12 @@ void choose_direct_geometry(Plan& p) {
         const int d = std::min(ndm - 1, t * 32 + l);
         // channels past the last read their own (zero) row at any delay
         const int32_t v = c < nchan ? p.delays[static_cast<size_t>(d) * nchan + c] : 0;
-        const uint32_t at = static_cast<uint32_t>((c % (64 * g.sgroups)) * g.cspan + (v >> 5) - b4);
-        p.dmeta[(static_cast<size_t>(t) * nc + c) * 32 + l] = (at * 4) << 5 | static_cast<uint32_t>(v & 31);
+        const size_t i = (static_cast<size_t>(t) * nc + c) * 32 + l;
+        const uint32_t word = static_cast<uint32_t>(c < nchan ? (v >> 5) - b4 : 0), shift = v & 31;
+        if (g.narrow)
+          p.dmeta[i / 2] |= (word << 5 | shift) << (16 * (i & 1));
+        else
+          p.dmeta[i] = ((c % (64 * g.sgroups)) * g.cspan + word) * 4 << 5 | shift;
       }
     }
   g.inst = inst;

@@ -161,7 +161,7 @@ extern "C" int snd_bind_workspace(snd_plan_t plan, void* d_ws, size_t bytes, voi
   dp.gmeta = at<uint32_t>(d_ws, o.gmeta);
   dp.tile_wb = at<int32_t>(d_ws, o.tile_wb);
   dp.delays = at<int32_t>(d_ws, o.delays);
-  dp.dmeta = at<uint32_t>(d_ws, o.dmeta);
+  dp.dmeta = at<void>(d_ws, o.dmeta);
   dp.dbase = at<int32_t>(d_ws, o.dbase);
   dp.level_fires = at<unsigned long long>(d_ws, o.level_fires);
   const bool z = p.mode == SND_MODE_ZFLOAT;

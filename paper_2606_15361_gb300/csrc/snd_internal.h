@@ -92,6 +92,7 @@ struct DirectGeom {
   int ndm_tiles = 0;     // ceil(ndm / 32)
   int cspan = 0;         // staged ring words per channel (multiple of 4)
   int sgroups = 1;       // 64-channel adder groups staged per round (1 or 2)
+  bool narrow = false;   // 16-bit table entries
   int smem_bytes = 0;
   int sub_lev = 0;       // graded: the exact level (first level whose nodes may exceed N)
   int sub_groups = 1;    // graded: 64-channel groups per exact-level node (the last may have fewer)
@@ -171,7 +172,7 @@ struct DevPtrs {
   int32_t* zeoff;          // zfloat: [ndm_tiles][nleaves + 1] first pattern of each (tile, leaf)
   int32_t* zent;           // zfloat: [patterns][8] window offset of each channel | (its first delay mod 8) << 28; [7]: leaf << 16 | span
   uint32_t* zdm;           // zfloat: [ndm_tiles][nleaves][16] pattern in the tile << 14 | delay past the pattern's first
-  uint32_t* dmeta;         // direct tree: [ndm_tiles][nchan][32] byte offset in a round's windows << 5 | shift
+  void* dmeta;             // direct tree: [ndm_tiles][nchan][32] window offset << 5 | shift, in 32 or 16 bits
   int32_t* dbase;          // direct tree: [ndm_tiles][nchan] first staged ring word (multiple of 4)
   unsigned long long* level_fires;  // [kMaxLevels] firing node-samples per tree level (SND_FLAG_LEVEL_RATES)
 };
@@ -237,7 +238,7 @@ struct Plan {
   TreeGeom geom{};
   DirectGeom dgeom{};
   bool direct = false;                  // the tree runs on the direct kernel (tree_direct.cu)
-  std::vector<uint32_t> dmeta;
+  std::vector<uint32_t> dmeta;          // (two 16-bit entries a word where dgeom.narrow)
   std::vector<int32_t> dbase;
   ZGeom zgeom{};
   std::vector<int32_t> zwb, zcarry, zeoff, zent;
@@ -340,10 +341,17 @@ struct GraphRunner {
 };
 
 cudaError_t launch_tree_z(const Plan& p, int64_t e_prev, int64_t e_new, void* d_plane_out, cudaStream_t s);
-// tree_direct.cu: the direct tree kernel of plans with p.direct
-cudaError_t launch_tree_direct(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream_t s);
-cudaError_t launch_tree_direct_batch(const Plan* const* plans, const int64_t* e_prev, const int64_t* e_new, int n,
-                                     cudaStream_t s);
+// tree_direct.cu, tree_direct16.cu: the direct tree kernel of plans with p.direct, for each width of the table
+// entries (DirectGeom::narrow)
+template <bool NARROW>
+cudaError_t launch_direct(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream_t s);
+template <bool NARROW>
+cudaError_t launch_direct_batch(const Plan* const* plans, const int64_t* e_prev, const int64_t* e_new, int n,
+                                cudaStream_t s);
+template <> cudaError_t launch_direct<false>(const Plan&, int64_t, int64_t, cudaStream_t);
+template <> cudaError_t launch_direct<true>(const Plan&, int64_t, int64_t, cudaStream_t);
+template <> cudaError_t launch_direct_batch<false>(const Plan* const*, const int64_t*, const int64_t*, int, cudaStream_t);
+template <> cudaError_t launch_direct_batch<true>(const Plan* const*, const int64_t*, const int64_t*, int, cudaStream_t);
 
 template <typename Stage>
 cudaError_t chunk_post(const Plan& p, const ChunkPos& c, void* d_plane_out, cudaStream_t s, Stage&& stage) {

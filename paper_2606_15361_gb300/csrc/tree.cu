@@ -992,7 +992,8 @@ cudaError_t launch_tree(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream
     p.launches += 1;
     return cudaGetLastError();
   }
-  if (p.direct) return launch_tree_direct(p, e_prev, e_new, s);
+  if (p.direct)
+    return p.dgeom.narrow ? launch_direct<true>(p, e_prev, e_new, s) : launch_direct<false>(p, e_prev, e_new, s);
   TreeArgs a;
   int ntx = 0;
   tree_args(p, e_prev, e_new, a, &ntx);
@@ -1019,7 +1020,9 @@ cudaError_t launch_tree_batch(const Plan* const* plans, const int64_t* e_prev, c
         den.push_back(e_new[i]);
       }
     if (!dp.empty()) {
-      const cudaError_t e = launch_tree_direct_batch(dp.data(), dep.data(), den.data(), static_cast<int>(dp.size()), s);
+      const int nd = static_cast<int>(dp.size());
+      cudaError_t e = launch_direct_batch<false>(dp.data(), dep.data(), den.data(), nd, s);
+      if (e == cudaSuccess) e = launch_direct_batch<true>(dp.data(), dep.data(), den.data(), nd, s);
       if (e != cudaSuccess) return e;
     }
   }

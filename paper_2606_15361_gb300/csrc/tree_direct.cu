@@ -22,9 +22,11 @@
 //    CTA's time tile (warp w: words w*KW ..), so per channel a lane reads one table entry and then
 //    KW+1 consecutive window words (a sliding funnel-shift window). An entry is the window's byte
 //    offset among the round's windows and the bit shift: one add gives the address, where a 16-bit
-//    word offset per channel took three instructions (25 -> 22 a channel and warp; tree 307 -> 295 us
+//    word offset per channel takes three instructions (25 -> 22 a channel and warp; tree 307 -> 295 us
 //    float, 345 -> 333 graded for 1024 channels x 2048 DMs x 16384 samples: the ALU pipe, 78% busy,
-//    bounds it). The 32 DMs of a tile read one channel at offsets that differ by less than 32 words,
+//    bounds it). 16-bit entries stay where their smaller table lets two CTAs share an SM and 32-bit
+//    ones do not: some coarse DM grids (see choose_direct_geometry). The file is compiled once for
+//    each (tree_direct16.cu). The 32 DMs of a tile read one channel at offsets that differ by less than 32 words,
 //    so the reads hit distinct banks (or broadcast) without conflicts.
 //  * channels are staged 64 or 128 at a time (a round): every warp issues TMA bulk copies
 //    (cp.async.bulk) of its share of the round's channel windows from the L2-resident bit
@@ -42,7 +44,16 @@
 namespace snd {
 namespace {
 
+#ifdef SND_DIRECT_NARROW
+constexpr bool kNarrow = true;
+using Entry = uint16_t;                          // (word offset in the channel's window << 5) | bit shift
+#else
+constexpr bool kNarrow = false;
+using Entry = uint32_t;                          // (byte offset in the round's windows << 5) | bit shift
+#endif
+
 constexpr int kDG = 64;                          // channels per adder group (one carry out)
+constexpr int kEntryRow = 32 * static_cast<int>(sizeof(Entry));  // table bytes of a channel
 constexpr long long kDirWaitCycles = kStageWaitCycles;
 
 struct DirArgs {
@@ -52,7 +63,7 @@ struct DirArgs {
   int level_nodes[kMaxLevels];
   int sub_groups;          // graded: staged groups per exact-level node
   int sub_lev;             // graded: the exact level
-  const uint32_t* meta;    // [ndm_tiles][nchan][32]: (byte offset in the round's windows << 5) | bit shift
+  const Entry* meta;       // [ndm_tiles][nchan][32]
   const int32_t* base4;    // [ndm_tiles][nchan]: first staged ring word (relative, multiple of 4)
   int cspan;               // staged words per channel (multiple of 4)
   int sgroups;             // adder groups of kDG channels staged per round (1 or 2)
@@ -584,8 +595,8 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
   const int SG = kDG * a.sgroups;                  // channels per staging round
   const int wbuf = SG * cspan;                     // window words per buffer
   uint32_t* win = sm;                              // [2][SG][cspan]
-  uint32_t* met = sm + 2 * wbuf;                   // [2][SG][32]
-  int32_t* sbase = reinterpret_cast<int32_t*>(sm + 2 * wbuf + 2 * SG * 32);  // [nchan]
+  Entry* met = reinterpret_cast<Entry*>(sm + 2 * wbuf);  // [2][SG][32]
+  int32_t* sbase = reinterpret_cast<int32_t*>(met + 2 * SG * 32);  // [nchan]
   const long long aw0 = a.word0 + static_cast<long long>(bx) * a.tile_words;
   const int lead = static_cast<int>(aw0 & 3);
   const long long aw4 = aw0 - lead;
@@ -615,7 +626,7 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     // the buffer's previous contents were read by every warp before the last barrier
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (lane == 0)
-      bar_expect(bar, static_cast<uint32_t>((i1 > i0 ? i1 - i0 : 0) * cspan * 4 + (wd == 0 ? SG * 128 : 0)));
+      bar_expect(bar, static_cast<uint32_t>((i1 > i0 ? i1 - i0 : 0) * cspan * 4 + (wd == 0 ? SG * kEntryRow : 0)));
     __syncwarp();
     for (int i = i0 + lane; i < i1; i += 32) {
       const int c = g * SG + i;
@@ -624,7 +635,7 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     }
     if (wd == 0 && lane == 0)
       bulk_g2s(smem_u32(met + b * SG * 32), a.meta + (static_cast<size_t>(tile) * a.nchan + g * SG) * 32,
-               static_cast<uint32_t>(SG * 128), bar);
+               static_cast<uint32_t>(SG * kEntryRow), bar);
   };
 
   DState<MODE, KW, NPL, MAXU> st;
@@ -642,12 +653,13 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
     if (ok && busy) {
 #pragma unroll 1
       for (int h = 0; h < a.sgroups; ++h) {
-        const uint32_t* M = met + b * SG * 32 + h * kDG * 32 + lane;
-        const uint32_t Wb = smem_u32(win + b * wbuf + lead + wd * KW);
+        const Entry* M = met + b * SG * 32 + h * kDG * 32 + lane;
+        // 16-bit offsets count from the channel's own window, 32-bit ones from the round's first
+        const uint32_t Wb = smem_u32(win + b * wbuf + (kNarrow ? h * kDG * cspan : 0) + lead + wd * KW);
         static_assert(KW == 2 || KW == 4, "window words per lane");
         auto fetch = [&](int ci, uint32_t (&v)[KW]) {
           const uint32_t m = M[ci * 32];
-          const uint32_t p = Wb + (m >> 5);
+          const uint32_t p = kNarrow ? Wb + static_cast<uint32_t>(ci * cspan) * 4u + (m >> 5) * 4u : Wb + (m >> 5);
           uint32_t x[KW + 1];
           x[0] = lds32<0>(p);
           x[1] = lds32<4>(p);
@@ -816,7 +828,7 @@ void direct_args(const Plan& p, int64_t e_prev, int64_t e_new, DirArgs& a, int* 
   for (int l = 0; l < kMaxLevels; ++l) a.level_nodes[l] = l < p.nlev ? p.level_nodes[l] : 1;
   a.sub_groups = g.sub_groups;
   a.sub_lev = g.sub_lev;
-  a.meta = dp.dmeta;
+  a.meta = static_cast<const Entry*>(dp.dmeta);
   a.base4 = dp.dbase;
   a.cspan = g.cspan;
   a.sgroups = g.sgroups;
@@ -836,7 +848,8 @@ void direct_args(const Plan& p, int64_t e_prev, int64_t e_new, DirArgs& a, int* 
 
 }  // namespace
 
-cudaError_t launch_tree_direct(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream_t s) {
+template <>
+cudaError_t launch_direct<kNarrow>(const Plan& p, int64_t e_prev, int64_t e_new, cudaStream_t s) {
   if (e_new <= e_prev) return cudaSuccess;
   DirArgs a;
   int ntx = 0;
@@ -861,9 +874,12 @@ cudaError_t launch_tree_direct(const Plan& p, int64_t e_prev, int64_t e_new, cud
   return dispatch_direct(g.rates_inst, gr);
 }
 
-cudaError_t launch_tree_direct_batch(const Plan* const* plans, const int64_t* e_prev, const int64_t* e_new, int n,
-                                     cudaStream_t s) {
+// (plans of the other entry width are passed over)
+template <>
+cudaError_t launch_direct_batch<kNarrow>(const Plan* const* plans, const int64_t* e_prev, const int64_t* e_new, int n,
+                                         cudaStream_t s) {
   std::vector<int> done(n, 0);
+  for (int i = 0; i < n; ++i) done[i] = plans[i]->dgeom.narrow != kNarrow;
   for (int i = 0; i < n; ++i) {
     if (done[i]) continue;
     const int key = plans[i]->dgeom.inst;
