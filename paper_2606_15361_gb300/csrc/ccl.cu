@@ -166,12 +166,6 @@ __device__ __forceinline__ void close_tile(const uint32_t* __restrict__ in, uint
   }
 }
 
-__global__ void __launch_bounds__(kCloseThreads) k_close(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                                         int ndm, int mw, int nb, int r) {
-  extern __shared__ uint32_t csm[];
-  close_tile(in, out, ndm, mw, nb, r, blockIdx.x, blockIdx.y, csm);
-}
-
 // One warp per row: number of runs (run starts) of the closed mask.
 __device__ __forceinline__ void run_count_row(const uint32_t* __restrict__ m, int ndm, int mw, int nb,
                                               int32_t* row_runs, const int warp, const int lane) {
@@ -795,18 +789,12 @@ cudaError_t launch_candidates(const Plan& p, int64_t f_prev, int nb, cudaStream_
   const int r = p.closing / 2;
   const int nbw = (nb + 31) / 32;
   dim3 blk(128), grd((nbw + 127) / 128, p.ndm);
-  if (r > 0 && (p.flags & kFlagReferenceTree)) {
-    // reference path: the four separable passes as separate launches
+  if (r > 0) {
     p.launches += 4;
     k_close_h<<<grd, blk, 0, s>>>(dp.mask, dp.mask2, p.mw, nb, r, 0);
     k_close_v<<<grd, blk, 0, s>>>(dp.mask2, dp.mask3, p.ndm, p.mw, nb, r, 0);
     k_close_h<<<grd, blk, 0, s>>>(dp.mask3, dp.mask2, p.mw, nb, r, 1);
     k_close_v<<<grd, blk, 0, s>>>(dp.mask2, dp.mask3, p.ndm, p.mw, nb, r, 1);
-  } else if (r > 0) {
-    p.launches += 1;
-    const int smem = 2 * (kCloseTR + 4 * r) * kCloseNQ * static_cast<int>(sizeof(uint32_t));
-    dim3 cg((nbw + kCloseTQ - 1) / kCloseTQ, (p.ndm + kCloseTR - 1) / kCloseTR);
-    k_close<<<cg, kCloseThreads, smem, s>>>(dp.mask, dp.mask3, p.ndm, p.mw, nb, r);
   } else {
     cudaMemcpyAsync(dp.mask3, dp.mask, sizeof(uint32_t) * static_cast<size_t>(p.ndm) * p.mw,
                     cudaMemcpyDeviceToDevice, s);
