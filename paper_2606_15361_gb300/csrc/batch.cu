@@ -2,11 +2,12 @@
 // and workspace), and one call advances all of them by one chunk each.
 //
 // Every stage of a step runs for all beams at once, in a fixed handful of launches:
-//  * the encoders: three launches (histogram, levels, pack) whose CTAs are spread over the
-//    beams by a prefix of their CTA counts;
+//  * the encoders: a launch per shared-memory class (at most three), whose clusters are spread
+//    over the beams by a prefix of their cluster counts (chunks too long for it: their own);
 //  * the trees: one persistent launch per kernel instantiation, whose resident CTAs take
 //    (beam, DM tile, time tile) work items from a device counter until none is left;
-//  * the matched filters: one launch, one CTA per (beam, DM row);
+//  * the matched filters: a launch per row shape (threads by the rows' length, at most four),
+//    one CTA per (beam, DM row);
 //  * the candidate stages: one cooperative launch whose stages are separated by bounded
 //    grid-wide barriers.
 // The per-beam arguments travel by value in each launch's parameter block. With graphs
@@ -37,7 +38,7 @@ int enqueue_plans(Plan* const* plans, int n, const uint8_t* const* d_chunks, con
   std::vector<ChunkPos> ppos;
   std::vector<int64_t> ep, en;
   for (int i = 0; i < n; ++i) pos[i] = chunk_pos(*plans[i], nsamp[i]);
-  // 1. every encoder (three launches for all bit-ring plans; each clears its block counters)
+  // 1. every encoder (a launch per shared-memory class; each clears its plan's block counters)
   if (launch_encode_batch(cp.data(), d_chunks, nsamp, n, s) != cudaSuccess) return SND_ERR_CUDA;
   // 2. the trees: one persistent launch per kernel instantiation
   for (int i = 0; i < n; ++i) {
@@ -55,7 +56,7 @@ int enqueue_plans(Plan* const* plans, int n, const uint8_t* const* d_chunks, con
   }
   if (!tp.empty() && launch_tree_batch(tp.data(), ep.data(), en.data(), static_cast<int>(tp.size()), s) != cudaSuccess)
     return SND_ERR_CUDA;
-  // 3. every matched filter in one launch, 4. every candidate stage in one cooperative launch
+  // 3. every matched filter (a launch per row shape), 4. every candidate stage in one cooperative launch
   for (int i = 0; i < n; ++i) {
     if (plans[i]->mode == SND_MODE_ZFLOAT) continue;
     post.push_back(plans[i]);

@@ -9,11 +9,12 @@
 //
 // Decision: a cell is in the mask iff max over the row's widths of
 //   SNR(W) = (S_W - mu*W) / (sigma*sqrt(W))          (FP64, this operation order)
-// reaches Theta. SNR(S) is monotone in the integer S, so thread 0 finds per width the
-// smallest integer tau_W with SNR(tau_W) >= Theta by a bounded search around
+// reaches Theta. SNR(S) is monotone in the integer S, so lane j of the last warp finds the
+// smallest integer tau_W with SNR(tau_W) >= Theta of width 2^j by a bounded search around
 // mu*W + Theta*sigma*sqrt(W); the per-cell test is then the exact integer compare
-// S_W >= tau_W. Cells in the mask get their FP64 S/N maximum (ties -> smaller width)
-// rounded to float and are appended to the block's cell list for peak selection.
+// S_W >= tau_W. Cells in the mask get their FP64 S/N maximum (ties -> smaller width; FP64 only
+// for the widths that FP32 leaves) rounded to float and are appended to the block's cell list
+// for peak selection.
 // Mode A floors sigma at sigma_min; Mode C scores the integer root counts (S/N does not
 // change under the 1/sqrt(N_f) scale).
 
@@ -362,8 +363,11 @@ __device__ __forceinline__ void mf_row(const MfArgs& a, const int d) {
       const int t = i + e;
       const uint32_t p0 = P[t];
       // The cell's S/N is the FP64 maximum over the widths. FP64 divides are slow here, so FP32 finds
-      // the widths that can hold it: S - floor(mu W) is an exact integer, and what is left rounds to
-      // a few 1e-7 of a value above Theta, so a width more than 1e-4 below the largest cannot.
+      // the widths that can hold it, those within 1e-4 of its own largest. That leaves no maximum out,
+      // whatever Theta is: FP32 gets x = S - mu W, an exact integer less a fraction, to 2^-25 and a
+      // relative 2^-22, which is below 4e-5 of an x from 2^-10 on. Where the largest S/N has a smaller x
+      // (at least 1 / nb, as mu is a multiple of that), x at any other width with a positive S/N is the
+      // same times the widths' ratio, and its S/N at least sqrt 2 below.
       float best32 = -3.0e38f;
 #pragma unroll
       for (int j = 0; j < kNumWidthSlots; ++j)

@@ -534,8 +534,10 @@ void choose_direct_geometry(Plan& p) {
   const int nchan = p.nchan, ndm = p.ndm;
   // the kernel adds 64 channels at a time: channels from nchan up to the next multiple are ring rows
   // that stay zero (a channel that never fires changes no sum and no quorum). Adding them costs less
-  // than the leaf-sharing kernel at every count: tree us per 8192 samples x 512 DMs, direct /
-  // leaf-sharing, graded B = 8: 8 channels 17 / 23, 65 19 / 52, 140 23 / 58, 300 30 / 93, 1000 58 / 207.
+  // than the leaf-sharing kernel: tree us per 8192 samples x 512 DMs, direct / leaf-sharing, graded
+  // B = 8: 8 channels 17 / 23, 65 19 / 52, 140 23 / 58, 300 30 / 93, 1000 58 / 207. Only calls that
+  // launch a few CTAs of at most half an adder group lose (128 DMs x 1024 samples: 12 channels 17 / 12,
+  // 33 16 / 14, 65 19 / 20).
   const int nc = static_cast<int>(align_up(nchan, 64));
   const bool rates = (p.flags & SND_FLAG_LEVEL_RATES) != 0;
   if (nc >= 8192 || (rates && nc != nchan)) return;

@@ -103,7 +103,7 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x989680;\n selp.u32 %0, 1, 0, p;\n}"
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 10000000;\n selp.u32 %0, 1, 0, p;\n}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
       : "memory");
@@ -1278,7 +1278,7 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   }
 }
 
-// (h, l) + x as an unevaluated FP32 pair: h + l keeps about 48 bits of a sum (error-free two-sum)
+// (h, l) + x as an unevaluated FP32 pair: h + l keeps about 48 bits of a sum (Knuth's error-free two-sum)
 __device__ __forceinline__ void pair_add(float& h, float& l, float x) {
   const float s = __fadd_rn(h, x);
   const float t = __fsub_rn(s, h);
@@ -1360,11 +1360,11 @@ __device__ __noinline__ void snippet_fp64(const float* __restrict__ plane, long 
 // column's 64 cells in registers, so the plane is read once, and with 64 loads in flight a
 // thread. The FP64 pipe of this chip runs 1/64 of the FP32 rate, so an FP64 evaluation per cell
 // bounds a kernel that should be bound by its stores: the sums, the differences v - mu and the
-// products with 1 / sd are unevaluated FP32 pairs (two-sum, two-product: about 48 bits, so the
-// rounded result is the FP64 one), FP64 only in one warp, for the CTA's two totals. The
+// products with 1 / sd are unevaluated FP32 pairs (Knuth's two-sum, Dekker's product with an FMA:
+// about 48 bits, so the result is the FP64 one to a rounding), FP64 only in one warp, for the CTA's two totals. The
 // deviations are summed about the mean, not as s2 / n - mu^2. 4096 snippets of a 2048 x 16384
-// plane take 200 us (64: 13 us); with FP64 sums and divisions per cell 1806 us (64: 72 us). What is left is latency: two CTAs fit an SM (the cells in registers), and each
-// loads, reduces twice and stores one after the other; the bytes alone would take about 80 us.
+// plane take 200 us (64: 13 us); with FP64 sums and divisions per cell 1806 us (64: 72 us). What is left
+// is latency: two CTAs fit an SM (the cells in registers), and each loads, reduces twice and stores one after the other; the bytes alone would take about 80 us.
 __global__ void __launch_bounds__(256, 2) k_snippets(const float* __restrict__ plane, long long ld, int ndm,
                                                      long long ncols, const int32_t* __restrict__ rows,
                                                      const int64_t* __restrict__ cols, int n,
