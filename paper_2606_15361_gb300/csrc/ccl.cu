@@ -837,7 +837,6 @@ cudaError_t launch_candidates_batch(const Plan* const* plans, const ChunkPos* po
   }
   for (size_t i0 = 0; i0 < batch.size(); i0 += kMaxCandBeams) {
     CandMulti m{};
-    int rmax = 0;
     for (size_t k = i0; k < batch.size() && m.nbeams < kMaxCandBeams; ++k) {
       const Plan& p = *plans[batch[k]];
       const ChunkPos& c = pos[batch[k]];
@@ -873,13 +872,13 @@ cudaError_t launch_candidates_batch(const Plan* const* plans, const ChunkPos* po
       m.first_rows[m.nbeams] = m.total_rows;
       m.total_close += ((nbw + kCloseTQ - 1) / kCloseTQ) * ((p.ndm + kCloseTR - 1) / kCloseTR);
       m.total_rows += (p.ndm + 7) / 8;
-      rmax = rmax > e.r ? rmax : e.r;
       ++m.nbeams;
     }
     const Plan& owner = *plans[batch[i0]];
     m.gbar = owner.dp.counters + kCntGridBar;
     m.wait_cycles = owner.wait_limit > 0 ? owner.wait_limit : kGridWaitCycles;
-    const int smem = std::max(2 * (kCloseTR + 4 * rmax) * kCloseNQ, 4 * kSmallRuns) * static_cast<int>(sizeof(uint32_t));
+    static_assert(2 * (kCloseTR + 4 * 15) * kCloseNQ <= 4 * kSmallRuns, "the widest closing's tile fits the join's shared memory");
+    constexpr int smem = 4 * kSmallRuns * static_cast<int>(sizeof(uint32_t));
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

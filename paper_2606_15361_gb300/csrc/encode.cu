@@ -622,7 +622,8 @@ bool enc_beam(const Plan& p, const uint8_t* chunk, int nsamp, int S, EncBeam& e)
 
 template <typename A>
 cudaError_t run_encode(void (*kern)(A), int threads, const A& args, int clusters, int S, int smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // the same value at every launch, as other threads may launch the kernel with other sizes
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncMaxSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(clusters) * S);

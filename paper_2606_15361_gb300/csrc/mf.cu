@@ -505,7 +505,7 @@ struct MfLaunch {
   cudaError_t go() {
     const void* kern = many ? reinterpret_cast<const void*>(k_mf_multi<NT>) : reinterpret_cast<const void*>(k_mf<NT>);
     int dev = 0, nsm = 0, per_sm = 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);

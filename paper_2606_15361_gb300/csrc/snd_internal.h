@@ -190,6 +190,11 @@ enum {
   kCntTaken = 16       // .. kCntTaken + kCntSlots: the counters as the last read took them
 };
 
+// The dynamic shared memory that the tree and matched-filter kernels are allowed (their static part is below
+// 3 KB). Set to the same value at every launch: were it the launch's own size, a thread that launches the kernel
+// for a smaller plan could take it from another between that one's setting and its launch.
+constexpr int kMaxDynSmem = 224 * 1024;
+
 // Where counters and the head of a candidate list, which follow each other on the device, are read back to
 // in one copy; candidates past kReadCands go to the caller's buffer in a second one. Pageable on purpose: a
 // page-locked buffer saves 3 to 9 us of an idle read (18 us against 21 to 27) and nothing that shows beside a

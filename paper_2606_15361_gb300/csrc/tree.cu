@@ -821,7 +821,7 @@ __global__ void k_tree_ref(RefArgs a) {
 template <int MODE, int MAXL, int KW, int TH, int DPW>
 cudaError_t run_tree(const TreeArgs& a, dim3 grid, dim3 block, int smem, cudaStream_t s) {
   auto kern = (a.C == 4 && a.nchan % 4 == 0) ? k_tree<MODE, MAXL, KW, TH, DPW, 4> : k_tree<MODE, MAXL, KW, TH, DPW, 0>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   kern<<<grid, block, smem, s>>>(a);
@@ -831,7 +831,7 @@ cudaError_t run_tree(const TreeArgs& a, dim3 grid, dim3 block, int smem, cudaStr
 template <int MODE, int MAXL, int KW, int TH, int DPW>
 cudaError_t run_tree_multi(const TreeMulti& m, int ct4, int nctas, dim3 block, int smem, cudaStream_t s) {
   auto kern = ct4 ? k_tree_multi<MODE, MAXL, KW, TH, DPW, 4> : k_tree_multi<MODE, MAXL, KW, TH, DPW, 0>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   kern<<<nctas, block, smem, s>>>(m);

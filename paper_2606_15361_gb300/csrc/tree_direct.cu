@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(256, 2) k_snd_multi(const __grid_constant__ Di
 template <int MODE, int KW, int NPL, int MAXU>
 cudaError_t run_direct(const DirArgs& a, dim3 grid, dim3 block, int smem, cudaStream_t s) {
   auto kern = k_snd<MODE, KW, NPL, MAXU>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e != cudaSuccess) return e;
   kern<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
@@ -757,7 +757,7 @@ cudaError_t run_direct(const DirArgs& a, dim3 grid, dim3 block, int smem, cudaSt
 template <int MODE, int KW, int NPL, int MAXU>
 cudaError_t run_direct_multi(const DirMulti& m, int ctas, dim3 block, int smem, cudaStream_t s) {
   auto kern = k_snd_multi<MODE, KW, NPL, MAXU>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   // persistent: as many CTAs as fit on the GPU at once (fewer if there are fewer items)
   int dev = 0, nsm = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);

@@ -262,7 +262,7 @@ template <typename ST, int MAXL, int NP>
 cudaError_t run_z(const ZArgs& a, dim3 grid, dim3 block, int smem, cudaStream_t s) {
   // the compile-time 4-channel leaf applies when every leaf has 4 channels
   auto kern = (a.C == 4 && a.nchan % 4 == 0) ? k_tree_z<ST, MAXL, NP, 4> : k_tree_z<ST, MAXL, NP, 0>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e != cudaSuccess) return e;
   kern<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(512, 1) k_tree_zs(const __grid_constant__ ZArg
 template <typename ST, int MAXL, int NP>
 cudaError_t run_zs(const ZArgs& a, dim3 grid, int smem, cudaStream_t s) {
   auto kern = (a.C == 4 && a.nchan % 4 == 0) ? k_tree_zs<ST, MAXL, NP, 4> : k_tree_zs<ST, MAXL, NP, 0>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e != cudaSuccess) return e;
   kern<<<grid, dim3(32, 16), smem, s>>>(a);
   return cudaGetLastError();
