@@ -483,10 +483,7 @@ extern "C" int snd_multirate_candidates(snd_multirate_t h, snd_candidate_t* host
   if (cudaGetLastError() != cudaSuccess) return fail(m, SND_ERR_CUDA);
   const uint32_t* hc = m.read.counters();
   const int head = static_cast<int>(std::min<int64_t>(std::min<int64_t>(cap, m.cap), snd::kReadCands));
-  if (cudaMemcpyAsync(m.read.buf, cnt, snd::kReadHead + sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    return fail(m, SND_ERR_CUDA);
+  if (snd::read_list(m.read, cnt, 1, false, head, s) != cudaSuccess) return fail(m, SND_ERR_CUDA);
   const int n = static_cast<int>(hc[1]);
   const int take = std::min(n, cap);
   if (take > 0) std::memcpy(host_out, m.read.cand(), sizeof(snd_candidate_t) * std::min(take, head));

@@ -34,6 +34,48 @@ void chunk_commit(Plan& p, const ChunkPos& c, int32_t nsamp, cudaStream_t s) {
   p.pending_host = -1;
 }
 
+namespace {
+
+// One CTA of 256 threads (see read_list); out_cand: null where the candidates are copied afterwards
+__global__ void __launch_bounds__(256) k_take(uint32_t* counters, int count_at, int reset, int head,
+                                              uint32_t* out, uint4* out_cand) {
+  __shared__ int n;
+  const int i = threadIdx.x;
+  if (i < kCntSlots) {
+    const uint32_t v = counters[i];
+    out[i] = v;
+    if (i == count_at) n = min(static_cast<int>(v), head);
+    if (reset && (i == count_at || i == count_at + 1)) counters[i] = 0;
+  }
+  if (!out_cand) return;
+  __syncthreads();
+  static_assert(sizeof(snd_candidate_t) == 32, "a candidate is two 16-byte words");
+  const uint4* cand = reinterpret_cast<const uint4*>(reinterpret_cast<unsigned char*>(counters) + kReadHead);
+  for (int k = i; k < 2 * n; k += 256) out_cand[k] = cand[k];
+}
+
+}  // namespace
+
+cudaError_t read_list(HostRead& r, uint32_t* counters, int count_at, bool reset, int head, cudaStream_t s) {
+  static_assert(kCntStatus == kCntCands + 1 && sizeof(uint32_t) * (kCntTaken + kCntSlots) <= kReadHead, "layout");
+  cudaError_t e = cudaSuccess;
+  if (r.direct < 0) {
+    int dev = 0, pageable = 0, tables = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev);
+    if (e != cudaSuccess) return e;
+    r.direct = pageable && tables;
+  }
+  uint32_t* out = r.direct ? reinterpret_cast<uint32_t*>(r.buf) : counters;
+  k_take<<<1, 256, 0, s>>>(counters, count_at, reset, head, out + kCntTaken,
+                           r.direct ? reinterpret_cast<uint4*>(r.buf + kReadHead) : nullptr);
+  e = cudaGetLastError();
+  if (e == cudaSuccess && !r.direct)
+    e = cudaMemcpyAsync(r.buf, counters, kReadHead + sizeof(snd_candidate_t) * head, cudaMemcpyDeviceToHost, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
 cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s) {
   if (take <= kReadCands) return cudaSuccess;
   const cudaError_t e = cudaMemcpyAsync(host_out + kReadCands, src + kReadCands,
@@ -70,13 +112,6 @@ cudaError_t mark(Plan& p, cudaStream_t s, size_t* slot) {
   }
   *slot = p.ev_used++;
   return cudaEventRecord(p.ev_pool[*slot], s);
-}
-
-// The counters go to their second copy, and the list's count and status word start afresh.
-__global__ void k_take_counters(uint32_t* counters) {
-  const int i = threadIdx.x;
-  counters[snd::kCntTaken + i] = counters[i];
-  if (i == snd::kCntCands || i == snd::kCntStatus) counters[i] = 0;
 }
 
 // Run one stage inside an NVTX range named for it (host-side enqueue time in a timeline
@@ -335,18 +370,11 @@ extern "C" int snd_candidates(snd_plan_t plan, snd_candidate_t* host_out, int32_
   Plan& p = *reinterpret_cast<Plan*>(plan);
   if (!p.bound) return SND_ERR_STATE;
   if (p.sticky) return p.sticky;
-  // the counters are taken and the list's count and status word reset before the copy is enqueued, so one
-  // wait covers all three
   cudaStream_t s = p.last_stream;
-  const uint32_t* cnt = p.read.counters() + snd::kCntTaken;
+  const uint32_t* cnt = p.read.counters();
   const int head = std::min(std::min(cap, p.cand_cap), snd::kReadCands);
-  k_take_counters<<<1, snd::kCntSlots, 0, s>>>(p.dp.counters);
   p.launches += 1;
-  if (cudaGetLastError() != cudaSuccess ||
-      cudaMemcpyAsync(p.read.buf, p.dp.counters, snd::kReadHead + sizeof(snd_candidate_t) * head,
-                      cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    return fail(p, SND_ERR_CUDA);
+  if (snd::read_list(p.read, p.dp.counters, snd::kCntCands, true, head, s) != cudaSuccess) return fail(p, SND_ERR_CUDA);
   const int n = static_cast<int>(cnt[snd::kCntCands]);
   const int take = n < cap ? n : cap;
   if (take > 0) std::memcpy(host_out, p.read.cand(), sizeof(snd_candidate_t) * std::min(take, head));

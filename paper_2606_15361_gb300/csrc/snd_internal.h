@@ -195,17 +195,22 @@ enum {
 // for a smaller plan could take it from another between that one's setting and its launch.
 constexpr int kMaxDynSmem = 224 * 1024;
 
-// Where counters and the head of a candidate list, which follow each other on the device, are read back to
-// in one copy; candidates past kReadCands go to the caller's buffer in a second one. Pageable on purpose: a
-// page-locked buffer saves 3 to 9 us of an idle read (18 us against 21 to 27) and nothing that shows beside a
-// chunk, but freeing it waits for all work on the GPU: destroying a plan took as long as other streams'
-// kernels (10 ms beside 20 matrix products; 7 us now), its first read 175 us (45 now).
+// Where counters and the head of a candidate list are read back to. Where the GPU reaches pageable memory
+// through the host's page tables (Grace), one kernel writes them here directly: a read is one launch and one
+// wait, 16 us idle; else they are copied, 21 us (the list follows the counters on the device). Neither needs
+// page-locked memory, with which a read took 18 us, but whose freeing waits for all work on the GPU, so that
+// destroying a plan took as long as other streams' kernels (10 ms beside 20 matrix products; 7 us now).
+// Candidates past kReadCands go to the caller's buffer in a copy of their own.
 constexpr int kReadCands = 512, kReadHead = 256;
 struct HostRead {
-  alignas(16) unsigned char buf[kReadHead + sizeof(snd_candidate_t) * kReadCands];
-  const uint32_t* counters() const { return reinterpret_cast<const uint32_t*>(buf); }
+  int direct = -1;  // whether the GPU may write to buf (-1: not asked yet)
+  alignas(16) unsigned char buf[kReadHead + sizeof(snd_candidate_t) * kReadCands] = {};  // touched by the host first
+  const uint32_t* counters() const { return reinterpret_cast<const uint32_t*>(buf) + kCntTaken; }
   const snd_candidate_t* cand() const { return reinterpret_cast<const snd_candidate_t*>(buf + kReadHead); }
 };
+// The kCntSlots counters and the first min(counters[count_at], head) candidates of the list behind them to r;
+// with `reset`, counters[count_at] and the status word after it start afresh. Waits for the stream.
+cudaError_t read_list(HostRead& r, uint32_t* counters, int count_at, bool reset, int head, cudaStream_t s);
 // The candidates [kReadCands, take) of the list at `src` (device) to host_out.
 cudaError_t read_tail(const snd_candidate_t* src, int take, snd_candidate_t* host_out, cudaStream_t s);
 
