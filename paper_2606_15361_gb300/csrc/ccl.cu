@@ -760,10 +760,8 @@ __global__ void __launch_bounds__(256) k_cand_multi(const __grid_constant__ Cand
   }
   if (!grid_barrier(m)) return;
   for (int b = 0; b < m.nbeams; ++b) {
-    // beam b's first candidates, mostly all it has, are CTA b's, so the beams' lists are ranked side by side
     const CandBeam& e = m.beam[b];
-    rank_items(e.bcand, e.cand, e.counters, e.cand_cap, e.ndm, e.f_prev, csm, (bid + nblk - b % nblk) % nblk * 256,
-               gthreads);
+    rank_items(e.bcand, e.cand, e.counters, e.cand_cap, e.ndm, e.f_prev, csm, bid * 256, gthreads);
   }
   if (!grid_barrier(m)) return;
   for (int b = gtid; b < m.nbeams; b += gthreads) bump(m.beam[b].counters, m.beam[b].cand_cap);
