@@ -596,7 +596,7 @@ __device__ __forceinline__ bool direct_cta(const DirArgs& a, int bx, int tile, u
   const int wbuf = SG * cspan;                     // window words per buffer
   uint32_t* win = sm;                              // [2][SG][cspan]
   Entry* met = reinterpret_cast<Entry*>(sm + 2 * wbuf);  // [2][SG][32]
-  int32_t* sbase = reinterpret_cast<int32_t*>(met + 2 * SG * 32);  // [nchan]
+  int32_t* sbase = reinterpret_cast<int32_t*>(sm + 2 * wbuf + 2 * SG * (kEntryRow / 4));  // [nchan]
   const long long aw0 = a.word0 + static_cast<long long>(bx) * a.tile_words;
   const int lead = static_cast<int>(aw0 & 3);
   const long long aw4 = aw0 - lead;
