@@ -465,8 +465,8 @@ __global__ void k_emit(const int32_t* row_runs, int ndm, int run_cap, const int3
 // Rank every block candidate by (t, dm_index) (keys are distinct: one peak pixel per island) and place it
 // after the candidates already held. Called by whole CTAs of 256 threads: a CTA takes the candidates
 // i0, i0 + stride, ... and the 255 after each, and brings the keys through shared memory (`keys`,
-// kRankTile words), from where four are compared per load. Read from the list itself, field by field, a
-// block of 1400 candidates took one CTA 0.5 ms, and one of 34,000 a small grid 3 ms.
+// kRankTile words), from where four are compared per load. Read from the list itself, field by field,
+// ranking 1446 candidates took one CTA 0.7 ms, and 34,000 a small grid 6.5 ms.
 constexpr int kRankTile = 2048;
 __device__ __forceinline__ void rank_items(const snd_candidate_t* bcand, snd_candidate_t* cand, uint32_t* counters,
                                            int cand_cap, int ndm, long long f_prev, uint32_t* keys, int i0,
@@ -644,7 +644,7 @@ __device__ __forceinline__ void join_small(const CandBeam& e, int n, uint32_t* c
 
 // What bounds it is latency: a few hundred runs and some ten thousand cells per block go through nine
 // dependent steps. So the grid is no larger than the block's tiles and rows need, one plan's short
-// serial steps (the scan, joining a small block's islands, the final list) run in the CTA that a barrier
+// serial steps (the scan, joining a small block's islands, a short final list) run in the CTA that a barrier
 // saw last, and the cells' peaks are reduced in the warp before their atomics. Stage times before and
 // after, us with the event pair (before: ten barriers of 304 CTAs and global walks): 128 x 1024 binary
 // 38 -> 29, 128 x 16384 65 -> 50, 2048 x 16384 binary 56 -> 48, graded 113 -> 66, float 81 -> 57; eight
